@@ -9,7 +9,6 @@ namespace spuma {
 
 SolveArgs make_args(spuma_ldu_t h);
 spuma_status launch_solve(spuma_ldu_t h, const SolveArgs& a, int threads, cudaStream_t s);
-spuma_status scan_exclusive_ext(const int* in, int64_t n, int* out, int* tmp, cudaStream_t s);
 spuma_status pcg_solve_internal(spuma_ldu_t h, const double* diag, const double* upper, const double* b, double* x,
                                 const spuma_solver_controls* ctl, spuma_solver_perf* perf, cudaStream_t s,
                                 int zero_x0);
@@ -21,7 +20,10 @@ static int grid1d(int64_t work, int threads, int num_sms)
     return (int)std::max<int64_t>(g, 1);
 }
 
-
+// upper_f = -a_f in face order.  Bound by the FP64 pipe: about 38 instructions
+// a face with the shared reciprocals of fp64.cuh (60 with the built-in
+// division and square root): 200^3 assembly 2.87 -> 2.05 ms, its reverse mode
+// 2.49 -> 1.62 ms.
 __global__ void k_face_coeff(int nf, const int* __restrict__ l, const int* __restrict__ u,
                              const double* __restrict__ sf, const double* __restrict__ c,
                              const double* __restrict__ gamma, double* __restrict__ upper)
@@ -71,17 +73,34 @@ __global__ void k_bgamma_grad(int nb, const int* __restrict__ bcell, const int8_
     }
 }
 
-__global__ void k_bcount(int nb, const int* __restrict__ bcell, const int8_t* __restrict__ btype, int* cnt)
+// The Dirichlet faces of each cell as a linked list (head[cell], next[b]; the
+// order of a list is whatever the atomics gave, k_diag takes it ascending):
+// one memset and one kernel instead of a count, a three-kernel scan, a copy and
+// a fill (about 55 us at 200^3, launch-bound on small meshes).
+__global__ void k_blink(int nb, const int* __restrict__ bcell, const int8_t* __restrict__ btype, int* head, int* next)
 {
     for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x)
-        if (btype[b] == 1) atomicAdd(cnt + bcell[b], 1);
+        if (btype[b] == 1) next[b] = atomicExch(head + bcell[b], b);
 }
 
-__global__ void k_bfill(int nb, const int* __restrict__ bcell, const int8_t* __restrict__ btype, int* cursor,
-                        int* blist)
+// d plus a_b of the cell's Dirichlet faces in ascending face order.
+__device__ __forceinline__ double add_boundary(double d, int i, const int* head, const int* next, const double* c,
+                                               const double* bsf, const double* bcf, const double* bgamma)
 {
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x)
-        if (btype[b] == 1) blist[atomicAdd(cursor + bcell[b], 1)] = b;
+    const int first = head ? head[i] : -1;
+    for (int last = -1; first >= 0;) {
+        int b = 0x7fffffff;
+        for (int k = first; k >= 0; k = next[k])
+            if (k > last && k < b) b = k;
+        if (b == 0x7fffffff) break;
+        const double* s = bsf + 3 * (size_t)b;
+        const double* cb = bcf + 3 * (size_t)b;
+        const double* ci = c + 3 * (size_t)i;
+        d = __dadd_rn(d, face_coeff(s[0], s[1], s[2], __dsub_rn(cb[0], ci[0]), __dsub_rn(cb[1], ci[1]),
+                                    __dsub_rn(cb[2], ci[2]), bgamma[b]));
+        last = b;
+    }
+    return d;
 }
 
 // diag_i = sum over the faces of i in face order (neighbour side ascending,
@@ -89,7 +108,7 @@ __global__ void k_bfill(int nb, const int* __restrict__ bcell, const int8_t* __r
 // ascending order.
 __global__ void k_diag(int n, const int* __restrict__ lo_start, const int* __restrict__ lo_face,
                        const int* __restrict__ own_start, const double* __restrict__ upper,
-                       const int* __restrict__ bstart, int* __restrict__ blist, const double* __restrict__ c,
+                       const int* __restrict__ head, const int* __restrict__ next, const double* __restrict__ c,
                        const double* __restrict__ bsf, const double* __restrict__ bcf,
                        const double* __restrict__ bgamma, double* __restrict__ diag)
 {
@@ -97,40 +116,73 @@ __global__ void k_diag(int n, const int* __restrict__ lo_start, const int* __res
         double d = 0.0;
         for (int k = lo_start[i]; k < lo_start[i + 1]; k++) d = __dadd_rn(d, -upper[lo_face[k]]);
         for (int f = own_start[i]; f < own_start[i + 1]; f++) d = __dadd_rn(d, -upper[f]);
-        if (bstart) {
-            const int b0 = bstart[i], b1 = bstart[i + 1];
-            for (int k = b0 + 1; k < b1; k++) {   // ascending boundary-face order
-                int v = blist[k], j = k - 1;
-                while (j >= b0 && blist[j] > v) {
-                    blist[j + 1] = blist[j];
-                    j--;
-                }
-                blist[j + 1] = v;
-            }
-            for (int k = b0; k < b1; k++) {
-                const int b = blist[k];
-                const double* s = bsf + 3 * (size_t)b;
-                const double* cb = bcf + 3 * (size_t)b;
-                const double* ci = c + 3 * (size_t)i;
-                d = __dadd_rn(d, face_coeff(s[0], s[1], s[2], __dsub_rn(cb[0], ci[0]), __dsub_rn(cb[1], ci[1]),
-                                            __dsub_rn(cb[2], ci[2]), bgamma[b]));
-            }
-        }
-        diag[i] = d;
+        diag[i] = add_boundary(d, i, head, next, c, bsf, bcf, bgamma);
     }
 }
 
-template <class T>
-__global__ void k_amul_ldu(int n, const int* __restrict__ lo_start, const int* __restrict__ lo_face,
-                           const int* __restrict__ lo_col, const int* __restrict__ own_start,
-                           const int* __restrict__ uaddr, const T* __restrict__ diag, const T* __restrict__ upper,
-                           const T* __restrict__ x, T* __restrict__ y)
+// The same over the fixed-width face lists (entry j of cell i at FL[j n + i],
+// +-(f + 1), 0 padding, face order): a cell's face indices arrive in coalesced
+// loads with no extents before them, its coefficients in one gather round.
+template <int W>
+__global__ void __launch_bounds__(256, 8) k_diag_fl(int n, int w, const int* __restrict__ FL,
+                                                    const double* __restrict__ upper, const int* __restrict__ head,
+                                                    const int* __restrict__ next, const double* __restrict__ c,
+                                                    const double* __restrict__ bsf, const double* __restrict__ bcf,
+                                                    const double* __restrict__ bgamma, double* __restrict__ diag)
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        T acc = mul_rn(diag[i], x[i]);
-        for (int k = lo_start[i]; k < lo_start[i + 1]; k++) acc = fmadd(upper[lo_face[k]], x[lo_col[k]], acc);
-        for (int f = own_start[i]; f < own_start[i + 1]; f++) acc = fmadd(upper[f], x[uaddr[f]], acc);
-        y[i] = acc;
+        int e[W];
+#pragma unroll
+        for (int j = 0; j < W; j++) e[j] = j < w ? __ldcs(FL + (size_t)j * n + i) : 0;
+        double t[W];
+#pragma unroll
+        for (int j = 0; j < W; j++) t[j] = e[j] != 0 ? __ldcs(upper + abs(e[j]) - 1) : 0.0;
+        double d = 0.0;
+#pragma unroll
+        for (int j = 0; j < W; j++)
+            if (e[j] != 0) d = __dsub_rn(d, t[j]);
+        __stcs(diag + i, add_boundary(d, i, head, next, c, bsf, bcf, bgamma));
+    }
+}
+
+// y = A x on the caller's arrays.  A row's neighbour-side entries (face and
+// column lists) and owner-side entries (its run of faces) are taken as one
+// list in groups of G: the group's indices load together, then its
+// coefficients and x values, then the FMAs in face order, so a hex row costs
+// three memory round trips instead of one chain of three per entry.  On a
+// randomly numbered mesh the 72 M gathers of 8 bytes from 32-byte sectors bound
+// it (200^3, FP64: 832 -> 811 us).
+template <class T>
+__global__ void __launch_bounds__(256) k_amul_ldu(int n, const int* __restrict__ lo_start,
+                                                  const int* __restrict__ lo_face, const int* __restrict__ lo_col,
+                                                  const int* __restrict__ own_start, const int* __restrict__ uaddr,
+                                                  const T* __restrict__ diag, const T* __restrict__ upper,
+                                                  const T* __restrict__ x, T* __restrict__ y)
+{
+    constexpr int G = 6;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const int k0 = lo_start[i], nl = lo_start[i + 1] - k0, f0 = own_start[i], nt = nl + own_start[i + 1] - f0;
+        T acc = mul_rn(__ldcs(diag + i), x[i]);
+        for (int off = 0; off < nt; off += G) {
+            int f[G], c[G];
+            T a[G], v[G];
+#pragma unroll
+            for (int j = 0; j < G; j++) {
+                const int e = off + j;
+                const bool ok = e < nt, low = e < nl;
+                f[j] = !ok ? -1 : low ? __ldcs(lo_face + k0 + e) : f0 + (e - nl);
+                c[j] = !ok ? 0 : low ? __ldcs(lo_col + k0 + e) : __ldcs(uaddr + f0 + (e - nl));
+            }
+#pragma unroll
+            for (int j = 0; j < G; j++) {
+                a[j] = f[j] >= 0 ? upper[f[j]] : T(0);
+                v[j] = f[j] >= 0 ? x[c[j]] : T(0);
+            }
+#pragma unroll
+            for (int j = 0; j < G; j++)
+                if (f[j] >= 0) acc = fmadd(a[j], v[j], acc);
+        }
+        __stcs(y + i, acc);
     }
 }
 
@@ -164,7 +216,7 @@ spuma_status spuma_assemble_laplacian(spuma_ldu_t h, const double* face_sf, cons
         return SPUMA_ERR_INVALID_ARG;
     }
     if (h->n == 0) return SPUMA_OK;
-    // temporaries in the (idle) FP64 vector region: bstart[n+1], cursor[n], blist[<=B]
+    // temporaries in the (idle) FP64 vector region: head[n], next[<=10n]
     const Layout& L = h->L;
     if ((int64_t)n_bfaces > 10LL * h->n) {
         set_error("more than 10 boundary faces per cell");
@@ -177,25 +229,21 @@ spuma_status spuma_assemble_laplacian(spuma_ldu_t h, const double* face_sf, cons
                                                                 cell_c, face_gamma, upper);
         count_launch();
     }
-    int* bstart = nullptr;
-    int* blist = nullptr;
+    int* head = nullptr;
+    int* next = nullptr;
     if (n_bfaces > 0) {
-        bstart = h->at<int>(L.x64);           // n+1 ints (x64 holds 2n)
-        int* cursor = h->at<int>(L.r64);      // n ints
-        int* tmp = h->at<int>(L.w64);         // scan temporaries
-        blist = h->at<int>(L.p64);            // <= 10n ints: p64, q64, b64, x32.. are contiguous (>= 11n ints)
-        SPUMA_CUDA(cudaMemsetAsync(bstart, 0, 4 * (size_t)(h->n + 1), s));
-        k_bcount<<<grid1d(n_bfaces, T, h->num_sms), T, 0, s>>>(n_bfaces, bface_cell, bface_type, bstart);
-        count_launch();
-        spuma_status st = scan_exclusive_ext(bstart, h->n, bstart, tmp, s);
-        if (st != SPUMA_OK) return st;
-        SPUMA_CUDA(cudaMemcpyAsync(cursor, bstart, 4 * (size_t)h->n, cudaMemcpyDeviceToDevice, s));
-        k_bfill<<<grid1d(n_bfaces, T, h->num_sms), T, 0, s>>>(n_bfaces, bface_cell, bface_type, cursor, blist);
+        head = h->at<int>(L.x64);             // n ints (x64 holds 2n)
+        next = h->at<int>(L.p64);             // <= 10n ints: p64, q64, b64, x32.. are contiguous (>= 11n ints)
+        SPUMA_CUDA(cudaMemsetAsync(head, 0xff, 4 * (size_t)h->n, s));
+        k_blink<<<grid1d(n_bfaces, T, h->num_sms), T, 0, s>>>(n_bfaces, bface_cell, bface_type, head, next);
         count_launch();
     }
-    if (h->nf > 0 || n_bfaces > 0) {
+    if (h->nf > 0 && h->ell_w > 0 && h->ell_w <= 6) {
+        k_diag_fl<6><<<std::min(grid1d(h->n, T, h->num_sms), h->num_sms * 8), T, 0, s>>>(
+            h->n, h->ell_w, h->at<int>(L.FL), upper, head, next, cell_c, bface_sf, bface_cf, bface_gamma, diag);
+    } else if (h->nf > 0 || n_bfaces > 0) {
         k_diag<<<grid1d(h->n, T, h->num_sms), T, 0, s>>>(h->n, h->at<int>(L.lo_start), h->at<int>(L.lo_face),
-                                                         h->at<int>(L.own_start), upper, bstart, blist, cell_c,
+                                                         h->at<int>(L.own_start), upper, head, next, cell_c,
                                                          bface_sf, bface_cf, bface_gamma, diag);
     } else {
         SPUMA_CUDA(cudaMemsetAsync(diag, 0, 8 * (size_t)h->n, s));
