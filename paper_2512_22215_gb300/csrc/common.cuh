@@ -161,32 +161,54 @@ __device__ __forceinline__ bool group_sync(const Group& g)
 // Block-level sums of NV doubles, written as this block's partials; after a
 // group_sync every block reads all partials of a slot in the same fixed order,
 // so the grid-wide result is deterministic and identical in every block.
+// GB300 issues an FP64 warp instruction per 64 cycles and SM quadrant: a
+// butterfly in all 32 warps of a block (five adds each) takes 40 of them per
+// quadrant, so the values meet in shared memory first and one warp per
+// quadrant adds up eight of them per lane (12 in all).  With the partials
+// below loaded together: one sum over the grid 2.7 -> 1.2 us by this count.
+__device__ __forceinline__ double* sum_buffer()   // one per kernel, whatever the NV of its sums
+{
+    __shared__ double buf[1024];
+    return buf;
+}
+template <int NV>
+__device__ __forceinline__ void block_sum_to_first(double (&v)[NV])   // result in thread 0
+{
+    double* buf = sum_buffer();
+    __shared__ double quad[4][NV];
+    const int tid = (int)threadIdx.x, bs = (int)blockDim.x, lane = tid & 31, warp = tid >> 5;
+    const int first = min(bs, 128);
+#pragma unroll
+    for (int k = 0; k < NV; k++) {
+        __syncthreads();
+        buf[tid] = v[k];
+        __syncthreads();
+        if (tid < first) {
+            double s = v[k];
+            for (int j = tid + 128; j < bs; j += 128) s += buf[j];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) quad[warp][k] = s;
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+#pragma unroll
+        for (int k = 0; k < NV; k++) {
+            double s = quad[0][k];
+            for (int w = 1; w < first >> 5; w++) s += quad[w][k];
+            v[k] = s;
+        }
+    }
+}
+
 template <int NV>
 __device__ __forceinline__ void block_reduce_store(double (&v)[NV], double* partials, int slot0, int bid)
 {
-    __shared__ double red[NV][32];
+    block_sum_to_first<NV>(v);
+    if (threadIdx.x == 0) {
 #pragma unroll
-    for (int k = 0; k < NV; k++) {
-        double s = v[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        v[k] = s;
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    __syncthreads();
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < NV; k++) red[k][warp] = v[k];
-    }
-    __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-        for (int k = 0; k < NV; k++) {
-            double s = lane < nw ? red[k][lane] : 0.0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) partials[(size_t)(slot0 + k) * kMaxBlocks + bid] = s;
-        }
+        for (int k = 0; k < NV; k++) partials[(size_t)(slot0 + k) * kMaxBlocks + bid] = v[k];
     }
 }
 
@@ -219,24 +241,41 @@ __device__ __forceinline__ void block_max_store(double (&v)[NV], double* partial
     }
 }
 
-// Grid-wide value of slot0..slot0+NV-1 (sum or max), broadcast to the block.
+// Grid-wide value of slot0..slot0+NV-1 (sum or max), broadcast to the block:
+// one warp takes every 32nd partial, five of each slot loaded together (152
+// blocks: all of them) before the first addition waits.
 template <int NV, bool MAX = false>
 __device__ __forceinline__ void grid_reduce_read(double (&out)[NV], const double* partials, int slot0, int nblocks)
 {
     __shared__ double bc[NV];
     const int lane = threadIdx.x & 31;
     if (threadIdx.x < 32) {
+        double s[NV];
 #pragma unroll
-        for (int k = 0; k < NV; k++) {
-            const volatile double* ps = partials + (size_t)(slot0 + k) * kMaxBlocks;
-            double s = 0.0;
-            for (int j = lane; j < nblocks; j += 32) s = MAX ? fmax(s, ps[j]) : s + ps[j];
+        for (int k = 0; k < NV; k++) s[k] = 0.0;
+        for (int b = lane; b < nblocks; b += 160) {
+            double t[NV][5];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                double t = __shfl_xor_sync(0xffffffffu, s, o);
-                s = MAX ? fmax(s, t) : s + t;
+            for (int k = 0; k < NV; k++)
+#pragma unroll
+                for (int j = 0; j < 5; j++)
+                    t[k][j] = b + 32 * j < nblocks ? __ldcg(partials + (size_t)(slot0 + k) * kMaxBlocks + b + 32 * j) : 0.0;
+#pragma unroll
+            for (int k = 0; k < NV; k++)
+#pragma unroll
+                for (int j = 0; j < 5; j++)
+                    if (b + 32 * j < nblocks) s[k] = MAX ? fmax(s[k], t[k][j]) : s[k] + t[k][j];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < NV; k++) {
+                const double t = __shfl_xor_sync(0xffffffffu, s[k], o);
+                s[k] = MAX ? fmax(s[k], t) : s[k] + t;
             }
-            if (lane == 0) bc[k] = s;
+        if (lane == 0) {
+#pragma unroll
+            for (int k = 0; k < NV; k++) bc[k] = s[k];
         }
     }
     __syncthreads();
