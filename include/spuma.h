@@ -516,10 +516,7 @@ int32_t spuma_tune_cache_store(const char* path, const char* signature, int32_t 
  * first block sweeps alone (0: none), SPUMA_SWEEP=0 strides a level's
  * rows over the blocks instead of giving each block one contiguous chunk of
  * every level, SPUMA_AMUL_CHUNKS=1 makes the PCG's Amul phase walk those
- * chunks too (on meshes whose levels are wide), and
- * SPUMA_GAMG_FUSE_SCALE_ROWS=n makes GAMG's coarse levels of at most n
- * cells apply the correction's scaling inside their first smoothing sweep
- * (0, the default: a pass of its own); SPUMA_GAMG_ORDER=inherited (read by
+ * chunks too (on meshes whose levels are wide); SPUMA_GAMG_ORDER=inherited (read by
  * spuma_gamg_create) stores GAMG's middle levels in the order inherited
  * from the level above instead of breadth-first.  With SPUMA_PHASE_CLOCKS a GAMG
  * solve fills the same table per V-cycle: 0..49 restriction into level

@@ -23,13 +23,14 @@
 // from 0 to 1e-8 relative; prolongation by injection, scaled by the A-norm
 // optimal step (e.r)/(e.Ae); two damped-Jacobi sweeps e += (2/3 rD)(r - Ae)
 // (or two two-stage Gauss-Seidel sweeps e += (D^-1 - D^-1 L D^-1)(r - A e)).
-// Levels of at most two rows per thread of one block run on the first block
-// alone with block-level barriers (the coarsest level's PCG on one warp when
-// it has at most 32 cells); the others on the whole grid.  Storage: level 0
-// in the mesh handle's internal (DIC level, Morton) order, the middle levels
+// Levels of at most kGamgSmall cells run on the first block alone with
+// block-level barriers (the coarsest level's PCG on one warp when it has at
+// most 32 cells); the others on the whole grid.  Storage: level 0 in the mesh
+// handle's internal (DIC level, Morton) order, the middle levels
 // breadth-first, the coarsest as built; rows and aggregates are moved, never
-// reordered inside, so every per-row sum follows the sequential definition's
-// order; dot products are deterministic block/grid reductions.
+// reordered inside.  Level 0's row sums follow the sequential definition's
+// order; a coarse row's entries are split over the four lanes of a team.
+// Every sum, the dot products included, is taken in a fixed order.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -49,6 +50,14 @@ constexpr int kGamgMaxLevels = 50;
 constexpr int kGamgCoarsest = 10;
 constexpr double kGamgOmega = 2.0 / 3.0;
 constexpr int kGamgPostSweeps = 2;
+// 512 threads leave 128 registers (the row teams' loads in flight; 1024 with
+// 64 spilled).  Levels of at most kGamgSmall cells on the first block: one SM's
+// FP64 pipe takes as long for a level of 700 cells (40 us, Gauss-Seidel) as the
+// whole grid with its barriers for one of 20 thousand; per V-cycle at 64^3
+// (Richardson) / 128^3 (Gauss-Seidel), limit 2048: 288 / 1370 us, 768: 270 /
+// 1321, 300: 261 / 1306, 100: 265 / 1310.
+constexpr int kGamgThreads = 512;
+constexpr int kGamgSmall = 300;
 constexpr double kGamgCoarseRelTol = 1e-8;
 enum GamgSlot { GS_A = 0, GS_B = 1, GS_C = 2, GS_D = 3 };   // reduction slots
 
@@ -59,6 +68,7 @@ struct GamgLevel {
     const int *rptr, *rcol, *rfac;          // row CSR for A_k: entries in ascending face order
     const int* rlo;                         // lower entries of each row (leading its entries)
     const int* agg;                         // cell -> next-level cell (k < L-1)
+    const int* cagg;                        // agg of each entry's column (row CSR; level 0: its fixed-width layout)
     const int *cptr, *ccell;                // next-level cell -> its cells (ascending)
     const int *fptr, *fface;                // next-level face -> its faces (ascending)
     const int *iptr, *iface;                // next-level cell -> the faces inside it (ascending)
@@ -101,12 +111,6 @@ struct GamgArgs {
     int max_iter, min_iter;
     double tol, rel_tol;
     long long* clk;                         // optional per-phase SM-clock totals of block 0 (diagnostics)
-    // coarse levels (k >= 1) of at most this many cells apply the correction's
-    // scaling inside their first smoothing sweep, each gathered e_j multiplied
-    // by the factor as it is read (the same rounded products as the scaled
-    // copy), one barrier step fewer; others keep the separate pass.  A
-    // measurement override (SPUMA_GAMG_FUSE_SCALE_ROWS), 0 by default.
-    int fuse_rows;
 };
 
 // --------------------------------------------------------------- device ---
@@ -131,16 +135,33 @@ struct GamgClock {
         }
     }
 };
+// Who takes the n items (rows, faces) of a step of level k: items first,
+// first + stride, ... below end, or (teams) the block's [c0, end).  A level of
+// the first block: that block's threads.  Coarse levels of the grid: one
+// contiguous chunk per block, a multiple of 32 items: GB300's FP64 pipe takes
+// one warp instruction per 64 cycles and quadrant, so a level of 6 thousand
+// rows handed out blockDim rows at a time keeps six SMs busy for 6 us per
+// Amul while the others wait (measured at 128^3, two-stage Gauss-Seidel: levels
+// of 100 to 3 thousand cells 82 -> 54 us each).  Level 0 strides its rows over
+// the grid when every thread has one (its chunks measured slower, 303 against
+// 338 us).
 struct Exec {
-    int first, stride;
+    int first, stride, c0, end;
     bool grid, active;
 };
 
-__device__ __forceinline__ Exec exec_for(const GamgArgs& a, int k, const Group& g)
+__device__ __forceinline__ Exec exec_grid(const Group& g, int n, bool strided)
 {
-    if (k >= a.small_from)
-        return Exec{(int)threadIdx.x, (int)blockDim.x, false, g.bid == 0};
-    return Exec{g.bid * (int)blockDim.x + (int)threadIdx.x, g.nblocks * (int)blockDim.x, true, true};
+    const int tid = (int)threadIdx.x, bs = (int)blockDim.x;
+    if (strided) return Exec{g.bid * bs + tid, g.nblocks * bs, 0, n, true, true};
+    const int chunk = ((n + g.nblocks - 1) / g.nblocks + 31) & ~31;
+    const int c0 = (int)min((long long)g.bid * chunk, (long long)n);
+    return Exec{c0 + tid, bs, c0, min(c0 + chunk, n), true, true};
+}
+__device__ __forceinline__ Exec exec_for(const GamgArgs& a, int k, const Group& g, int n)
+{
+    if (k >= a.small_from) return Exec{(int)threadIdx.x, (int)blockDim.x, 0, n, false, g.bid == 0};
+    return exec_grid(g, n, k == 0 && n >= g.nblocks * (int)blockDim.x);
 }
 
 // Barrier after a step done with `x`: the grid barrier, or the first block's
@@ -165,29 +186,11 @@ __device__ __forceinline__ bool exec_sum(const Exec& x, double (&v)[NV], const G
     }
     if (g.bid != 0) return true;
     // the first block alone: the same sums through shared memory only
-    __shared__ double red[NV][32];
     __shared__ double bc[NV];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    block_sum_to_first<NV>(v);
+    if (threadIdx.x == 0)
 #pragma unroll
-    for (int k = 0; k < NV; k++) {
-        double s = v[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        v[k] = s;
-    }
-    __syncthreads();
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < NV; k++) red[k][warp] = v[k];
-    __syncthreads();
-    if (warp == 0)
-#pragma unroll
-        for (int k = 0; k < NV; k++) {
-            double s = lane < nw ? red[k][lane] : 0.0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) bc[k] = s;
-        }
+        for (int k = 0; k < NV; k++) bc[k] = v[k];
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < NV; k++) v[k] = bc[k];
@@ -257,73 +260,150 @@ __device__ __forceinline__ double lvl0_amul_row(const GamgLvl0& z, X x, int p)
     return y;
 }
 
-// A level's row operations, in internal order at level 0 when z.on.
-__device__ __forceinline__ double level_amul_row(const GamgArgs& a, int k, const double* x, int i)
+// (A_0 x)_i for the outer residual (internal order when z.on).
+__device__ __forceinline__ double level0_amul_row(const GamgArgs& a, const double* x, int i)
 {
-    auto xv = [x](int c) { return x[c]; };
-    if (k == 0 && a.z.on) return lvl0_amul_row(a.z, xv, i);
-    return gamg_amul_row_g(a.lv[k], a.lv[k].diag, xv, i);
+    if (a.z.on) return lvl0_amul_row(a.z, [x](int c) { return x[c]; }, i);
+    return gamg_amul_row(a.lv[0], a.lv[0].diag, x, i);
 }
 
-// Rows first, first + stride, ... of level k: body(i, (A_k x)_i, x_i, U_i,
-// V_i) (U, V: the pass's own per-row inputs; NULL reads 0).  Level 0 in
-// internal order with a fixed-width layout of at most 6 entries is
-// software-pipelined: the next row's columns are loaded before this row's
-// gathers, and this row's coefficients, x, diagonal, U and V load beside its
-// gathers, so a row costs about one memory round trip; its sum is the same
-// FMA chain as lvl0_amul_row's.  Measured at 200^3 (face-area Richardson):
-// level 0's passes 948 -> 785 us per V-cycle; the same for the outer residual
-// pass, and the next row's extents one row ahead on the row-CSR levels, were
-// slower and are not used.
+// Level 0's rows first, first + stride, ... below n: body(p, (A_0 x)_p, x_p,
+// U_p, V_p) for the vector x_c = v[cols(c)] (U, V: the pass's own per-row
+// inputs; NULL reads 0).  `cols`: the entries' indices into v in the
+// fixed-width layout (the columns, or the columns' aggregates), `own`: a row's
+// own index into v (NULL: the row itself).  With a layout of at most 6
+// entries the rows are software-pipelined: the next row's indices are loaded
+// before this row's gathers, and this row's coefficients, x, diagonal, U and
+// V load beside its gathers, so a row costs about one memory round trip; its
+// sum is the same FMA chain as lvl0_amul_row's.  Measured at 200^3
+// (face-area Richardson): level 0's passes 948 -> 785 us per V-cycle.
 template <class Body>
-__device__ __forceinline__ void level_rows(const GamgArgs& a, int k, const double* x, const double* U,
-                                           const double* V, int first, int stride, Body body)
+__device__ __forceinline__ void lvl0_rows(const GamgLvl0& z, const int* cols, const int* own, const double* v,
+                                          const double* U, const double* V, int first, int stride, int n, Body body)
 {
-    const int n = a.lv[k].n;
-    if (k == 0 && a.z.on && a.z.ell_w > 0 && a.z.ell_w <= 6) {
-        const GamgLvl0& z = a.z;
-        auto cols = [&](int (&c)[6], int p) {
+    if (z.ell_w > 0 && z.ell_w <= 6) {
+        auto load = [&](int (&c)[6], int p) {
 #pragma unroll
-            for (int j = 0; j < 6; j++) c[j] = j < z.ell_w ? __ldcs(z.Ecol + (size_t)j * z.n + p) : -1;
+            for (int j = 0; j < 6; j++) c[j] = j < z.ell_w ? __ldcs(cols + (size_t)j * z.n + p) : -1;
         };
         int cur[6];
-        if (first < n) cols(cur, first);
+        if (first < n) load(cur, first);
         for (int p = first; p < n; p += stride) {
             int nxt[6];
             const int pn = p + stride;
-            if (pn < n) cols(nxt, pn);
+            if (pn < n) load(nxt, pn);
             double g6[6];
 #pragma unroll
-            for (int j = 0; j < 6; j++) g6[j] = cur[j] >= 0 ? x[cur[j]] : 0.0;
-            const double xp = x[p], d = __ldcs(z.d + p);
-            const double u = U ? U[p] : 0.0, v = V ? V[p] : 0.0;
+            for (int j = 0; j < 6; j++) g6[j] = cur[j] >= 0 ? v[cur[j]] : 0.0;
+            const double xp = v[own ? own[p] : p], d = __ldcs(z.d + p);
+            const double u = U ? U[p] : 0.0, w = V ? V[p] : 0.0;
             double y = __dmul_rn(d, xp);
 #pragma unroll
             for (int j = 0; j < 6; j++)
                 if (cur[j] >= 0) y = __fma_rn(__ldcs(z.Ea + (size_t)j * z.n + p), g6[j], y);
-            body(p, y, xp, u, v);
+            body(p, y, xp, u, w);
 #pragma unroll
             for (int j = 0; j < 6; j++) cur[j] = nxt[j];
         }
         return;
     }
-    for (int i = first; i < n; i += stride) {
-        const double u = U ? U[i] : 0.0, v = V ? V[i] : 0.0;
-        body(i, level_amul_row(a, k, x, i), x[i], u, v);
+    auto x = [v, own](int c) { return v[own ? own[c] : c]; };
+    for (int p = first; p < n; p += stride) {
+        const double u = U ? U[p] : 0.0, w = V ? V[p] : 0.0;
+        body(p, lvl0_amul_row(z, x, p), x(p), u, w);
     }
 }
 
-// s - sum over the row's lower entries (face order) of a_f y_col, one FMA each
-// (the two-stage Gauss-Seidel's second stage).
-__device__ __forceinline__ double level_lower_sweep(const GamgArgs& a, int k, const double* y, int i, double s)
+// Coarse rows [c0, end) of one block by teams of four lanes: body(i, sum over
+// the row's entries, the first cnt_i of them when cnt is given, of val_e
+// v[col_e]), called on one lane per row.  A team's lanes take every fourth
+// entry (neighbouring lanes read neighbouring entries) and add up in a fixed
+// order.  RT rows per team: 4 on levels that fill the block, where the lanes
+// then hold one finished row each (three adds for four rows, and the body runs
+// on every lane); 1 below, for the shorter chain.  A warp's FP64 instruction
+// takes its quadrant's pipe for 64 cycles however many lanes are live: a
+// thread per row pays for the longest of 32 rows (20 to 25 entries against 9
+// to 15 on average), one entry after the other.
+template <int RT, class Body>
+__device__ __forceinline__ void team_rows_t(const int* rptr, const int* cnt, const int* col, const double* val,
+                                            const double* v, int c0, int end, Body body)
 {
-    if (k == 0 && a.z.on) {
-        for (int e = a.z.Lptr[i]; e < a.z.Lptr[i + 1]; e++) s = __fma_rn(-a.z.La[e], y[a.z.Lcol[e]], s);
-        return s;
+    static_assert(RT == 1 || RT == 4, "rows per team");
+    constexpr int G = RT == 1 ? 4 : 2;      // entries per lane and load group
+    const int t = (int)threadIdx.x & 3, per = ((int)blockDim.x >> 2) * RT;
+    for (int base = c0; base < end; base += per) {
+        const int i0 = base + ((int)threadIdx.x >> 2) * RT;
+        double s[RT];
+        int e[RT], e1[RT];
+#pragma unroll
+        for (int k = 0; k < RT; k++) {
+            const bool ok = i0 + k < end;
+            const int b = ok ? rptr[i0 + k] : 0;
+            e1[k] = ok ? (cnt ? b + cnt[i0 + k] : rptr[i0 + k + 1]) : 0;
+            e[k] = b + t;
+            s[k] = 0.0;
+        }
+        for (;;) {
+            bool more = false;
+#pragma unroll
+            for (int k = 0; k < RT; k++) more |= e[k] < e1[k];
+            if (!more) break;
+            int c[RT][G];
+            double a[RT][G], x[RT][G];
+#pragma unroll
+            for (int k = 0; k < RT; k++)
+#pragma unroll
+                for (int j = 0; j < G; j++) {
+                    const bool ok = e[k] + 4 * j < e1[k];
+                    c[k][j] = ok ? __ldg(col + e[k] + 4 * j) : -1;
+                    a[k][j] = ok ? val[e[k] + 4 * j] : 0.0;
+                }
+#pragma unroll
+            for (int k = 0; k < RT; k++)
+#pragma unroll
+                for (int j = 0; j < G; j++) x[k][j] = c[k][j] >= 0 ? v[c[k][j]] : 0.0;
+#pragma unroll
+            for (int k = 0; k < RT; k++) {
+#pragma unroll
+                for (int j = 0; j < G; j++)
+                    if (c[k][j] >= 0) s[k] = __fma_rn(a[k][j], x[k][j], s[k]);
+                e[k] += 4 * G;
+            }
+        }
+        __syncwarp();
+        if (RT == 1) {
+            double r = s[0];
+            r = __dadd_rn(r, __shfl_xor_sync(0xffffffffu, r, 1));
+            r = __dadd_rn(r, __shfl_xor_sync(0xffffffffu, r, 2));
+            if (t == 0 && i0 < end) body(i0, r);
+        } else {
+            // lane t ends with row i0 + t: rows of its parity first, then its half
+            const bool odd = t & 1, high = t & 2;
+            double lo = odd ? s[1 % RT] : s[0], lo_out = odd ? s[0] : s[1 % RT];
+            double hi = odd ? s[3 % RT] : s[2 % RT], hi_out = odd ? s[2 % RT] : s[3 % RT];
+            lo = __dadd_rn(lo, __shfl_xor_sync(0xffffffffu, lo_out, 1));
+            hi = __dadd_rn(hi, __shfl_xor_sync(0xffffffffu, hi_out, 1));
+            const double keep = high ? hi : lo, out = high ? lo : hi;
+            const double r = __dadd_rn(keep, __shfl_xor_sync(0xffffffffu, out, 2));
+            if (i0 + t < end) body(i0 + t, r);
+        }
     }
-    const GamgLevel& L = a.lv[k];
-    const int e0 = L.rptr[i], e1 = e0 + L.rlo[i];
-    for (int e = e0; e < e1; e++) s = __fma_rn(-L.rval[e], y[L.rcol[e]], s);
+}
+template <class Body>
+__device__ __forceinline__ void team_rows(const GamgLevel& L, const int* cnt, const int* col, const double* v,
+                                          const Exec& x, Body body)
+{
+    if (x.end - x.c0 > (int)blockDim.x / 2)
+        team_rows_t<4>(L.rptr, cnt, col, L.rval, v, x.c0, x.end, body);
+    else
+        team_rows_t<1>(L.rptr, cnt, col, L.rval, v, x.c0, x.end, body);
+}
+
+// s - sum over level 0's lower entries (face order) of a_f y_col, one FMA each
+// (the two-stage Gauss-Seidel's second stage).
+__device__ __forceinline__ double lvl0_lower_sweep(const GamgLvl0& z, const double* y, int i, double s)
+{
+    for (int e = z.Lptr[i]; e < z.Lptr[i + 1]; e++) s = __fma_rn(-z.La[e], y[z.Lcol[e]], s);
     return s;
 }
 
@@ -354,15 +434,16 @@ __device__ bool gamg_coarse_matrices(const GamgArgs& a, const Group& g)
     if (a.z.on) lvl0_gather(a, g.bid * (int)blockDim.x + (int)threadIdx.x, g.nblocks * (int)blockDim.x);
     for (int k = 0; k + 1 < a.nlev; k++) {
         const GamgLevel& F = a.lv[k];
-        const Exec x = exec_for(a, k + 1, g);
+        const int nfc = a.lv[k + 1].nf, nc = a.lv[k + 1].n;
+        const Exec x = exec_for(a, k + 1, g, nc);
         if (x.active) {
-            const int nfc = a.lv[k + 1].nf, nc = a.lv[k + 1].n;
-            for (int c = x.first; c < nfc; c += x.stride) {
+            const Exec xf = exec_for(a, k + 1, g, nfc);
+            for (int c = xf.first; c < xf.end; c += xf.stride) {
                 double s = 0.0;
                 for (int j = F.fptr[c]; j < F.fptr[c + 1]; j++) s = __dadd_rn(s, F.upper[F.fface[j]]);
                 F.cupper[c] = s;
             }
-            for (int c = x.first; c < nc; c += x.stride) {
+            for (int c = x.first; c < x.end; c += x.stride) {
                 double s = 0.0;
                 for (int j = F.cptr[c]; j < F.cptr[c + 1]; j++) s = __dadd_rn(s, F.diag[F.ccell[j]]);
                 for (int j = F.iptr[c]; j < F.iptr[c + 1]; j++) s = __dadd_rn(s, __dmul_rn(2.0, F.upper[F.iface[j]]));
@@ -429,82 +510,94 @@ __device__ void gamg_dic_seq(const GamgLevel& L, const double* rD, const double*
     }
 }
 
-// Sum over the warp's lanes (a butterfly: every lane gets the same value,
-// the same sum as the first block's reduction when only warp 0 holds values).
-__device__ __forceinline__ double warp_sum(double s)
+// Sum over the first `width` lanes (a power of two; the other lanes hold
+// zeros or sums of their own): a butterfly, every lane gets its value.
+__device__ __forceinline__ double warp_sum(double s, int width)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    for (int o = width >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     return s;
 }
 
-// The coarsest level's PCG on warp 0 of the first block, one row per lane
-// (levels of at most 32 cells, the usual case): the same steps and sums as
-// gamg_coarsest below, with warp barriers instead of block barriers.
-__device__ void gamg_coarsest_warp(const GamgArgs& a, const GamgLevel& L)
+// The coarsest level's matrix for the warp PCG below, dense in shared memory
+// (column j's coefficients at 32 j; zeros off the pattern) with 1/diag, filled
+// once per solve by the first block.
+struct CoarseDense {
+    double a[32 * 32], rd[32];
+};
+
+__device__ void gamg_coarse_dense(const GamgLevel& L, CoarseDense& D)
 {
+    for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x) D.a[e] = 0.0;
+    __syncthreads();
     const int i = (int)threadIdx.x;
-    const bool row = i < L.n;
-    double* e = L.e;
-    double* r = a.pw;
-    double *w = a.pq, *p = a.pp, *q = a.px;
-    double ri = row ? L.r[i] : 0.0;
-    if (row) {
-        e[i] = 0.0;
-        r[i] = ri;
+    if (i < L.n) {
+        D.a[32 * i + i] = L.diag[i];
+        D.rd[i] = __ddiv_rn(1.0, L.diag[i]);
+        for (int e = L.rptr[i]; e < L.rptr[i + 1]; e++) D.a[32 * L.rcol[e] + i] = L.rval[e];
     }
-    const double v0 = warp_sum(row ? fabs(ri) : 0.0);
-    const double nfac = v0 + 1e-20;
-    const double res0 = v0 / nfac;
-    double res = res0, rho = 1.0, rho_old;
-    const int max_it = 2 * L.n + 10;
+    __syncthreads();
+}
+
+// The coarsest level's PCG on warp 0 of the first block, one row per lane
+// (levels of at most 32 cells, the usual case): the same steps as
+// gamg_coarsest below, the vectors in registers, p handed round by shuffles.
+// One warp issues an FP64 instruction per 64 cycles, so what counts is their
+// number: the sums run over as many lanes as the level needs, and the tests
+// compare products (|s| < 1e-300 nfac, sum|r| < tol sum|r0|) instead of
+// dividing (9 instructions each): 33 -> 15 us per V-cycle at 64^3.
+__device__ void gamg_coarsest_warp(const GamgArgs& a, const GamgLevel& L, const CoarseDense& D)
+{
+    const int i = (int)threadIdx.x, n = L.n;
+    const bool row = i < n;
+    int width = 1;
+    while (width < n) width <<= 1;
+    const double rd = row ? D.rd[i] : 0.0;
+    double ri = row ? L.r[i] : 0.0, ei = 0.0, pi = 0.0;
+    // every sum is taken from lane 0's group, so that all lanes see one value
+    // and leave the loop together (its shuffles name the whole warp)
+    double m = __shfl_sync(0xffffffffu, warp_sum(fabs(ri), width), 0);
+    const double stop = kGamgCoarseRelTol * m, tiny = 1e-300 * (m + 1e-20);
+    double rho = 1.0, rho_old;
+    const int max_it = 2 * n + 10;
     int it = 0;
-    if (res0 > 0.0) {
+    if (m > 0.0) {
         do {
             rho_old = rho;
-            double wi = 0.0;
+            double wi;
             if (a.coarsest_precond == SPUMA_PRECOND_DIC) {
+                if (row) a.pw[i] = ri;
                 __syncwarp();
-                if (i == 0) gamg_dic_seq(L, a.crD, r, w);
+                if (i == 0) gamg_dic_seq(L, a.crD, a.pw, a.pq);
                 __syncwarp();
-                if (row) wi = w[i];
-            } else if (row) {
-                wi = __dmul_rn(__ddiv_rn(1.0, L.diag[i]), ri);
-                w[i] = wi;
+                wi = row ? a.pq[i] : 0.0;
+            } else {
+                wi = __dmul_rn(rd, ri);
             }
-            rho = warp_sum(row ? __fma_rn(wi, ri, 0.0) : 0.0);
-            const double beta = it == 0 ? 0.0 : rho / rho_old;
-            if (row) p[i] = it == 0 ? wi : __fma_rn(beta, p[i], wi);
-            __syncwarp();
+            rho = __shfl_sync(0xffffffffu, warp_sum(__dmul_rn(wi, ri), width), 0);
+            pi = it == 0 ? wi : __fma_rn(rho / rho_old, pi, wi);
             double qi = 0.0;
-            if (row) {
-                qi = gamg_amul_row(L, L.diag, p, i);
-                q[i] = qi;
-            }
-            const double s = warp_sum(row ? __fma_rn(qi, p[i], 0.0) : 0.0);
-            if (fabs(s) / nfac < 1e-300) break;
+            for (int j = 0; j < n; j++) qi = __fma_rn(D.a[32 * j + i], __shfl_sync(0xffffffffu, pi, j), qi);
+            const double s = __shfl_sync(0xffffffffu, warp_sum(__dmul_rn(qi, pi), width), 0);
+            if (fabs(s) < tiny) break;
             const double alpha = rho / s;
-            if (row) {
-                e[i] = __fma_rn(alpha, p[i], e[i]);
-                ri = __fma_rn(-alpha, qi, ri);
-                r[i] = ri;
-            }
-            res = warp_sum(row ? fabs(ri) : 0.0) / nfac;
-            __syncwarp();
-        } while (++it < max_it && !(res < kGamgCoarseRelTol * res0));
+            ei = __fma_rn(alpha, pi, ei);
+            ri = __fma_rn(-alpha, qi, ri);
+            m = __shfl_sync(0xffffffffu, warp_sum(fabs(ri), width), 0);
+        } while (++it < max_it && !(m < stop));
     }
+    if (row) L.e[i] = ei;
 }
 
 // Coarsest level: PCG with the diagonal preconditioner from 0, relative
 // tolerance kGamgCoarseRelTol, at most 2n + 10 iterations (PCG recurrences).
-__device__ bool gamg_coarsest(const GamgArgs& a, const Group& g)
+__device__ bool gamg_coarsest(const GamgArgs& a, const Group& g, const CoarseDense& D)
 {
     const int k = a.nlev - 1;
     const GamgLevel& L = a.lv[k];
-    const Exec x = exec_for(a, k, g);
+    const Exec x = exec_for(a, k, g, L.n);
     if (!x.active) return true;   // the coarsest level is the first block's alone
     if (!x.grid && L.n <= 32) {
-        if (threadIdx.x < 32) gamg_coarsest_warp(a, L);
+        if (threadIdx.x < 32) gamg_coarsest_warp(a, L, D);
         return exec_sync(x, g);
     }
     double* e = L.e;
@@ -512,7 +605,7 @@ __device__ bool gamg_coarsest(const GamgArgs& a, const Group& g)
     double *w = a.pq, *p = a.pp, *q = a.px;
     double v[1] = {0.0};
     if (x.active)
-        for (int i = x.first; i < L.n; i += x.stride) {
+        for (int i = x.first; i < x.end; i += x.stride) {
             e[i] = 0.0;
             r[i] = L.r[i];
             v[0] += fabs(L.r[i]);
@@ -530,9 +623,9 @@ __device__ bool gamg_coarsest(const GamgArgs& a, const Group& g)
             if (a.coarsest_precond == SPUMA_PRECOND_DIC) {
                 if (g.bid == 0 && threadIdx.x == 0) gamg_dic_seq(L, a.crD, r, w);
                 if (!exec_sync(x, g)) return false;
-                for (int i = x.first; i < L.n; i += x.stride) t[0] = __fma_rn(w[i], r[i], t[0]);
+                for (int i = x.first; i < x.end; i += x.stride) t[0] = __fma_rn(w[i], r[i], t[0]);
             } else {
-                for (int i = x.first; i < L.n; i += x.stride) {
+                for (int i = x.first; i < x.end; i += x.stride) {
                     const double wi = __dmul_rn(__ddiv_rn(1.0, L.diag[i]), r[i]);
                     w[i] = wi;
                     t[0] = __fma_rn(wi, r[i], t[0]);
@@ -542,11 +635,11 @@ __device__ bool gamg_coarsest(const GamgArgs& a, const Group& g)
             rho = t[0];
             const double beta = it == 0 ? 0.0 : rho / rho_old;
             if (x.active)
-                for (int i = x.first; i < L.n; i += x.stride) p[i] = it == 0 ? w[i] : __fma_rn(beta, p[i], w[i]);
+                for (int i = x.first; i < x.end; i += x.stride) p[i] = it == 0 ? w[i] : __fma_rn(beta, p[i], w[i]);
             if (!exec_sync(x, g)) return false;
             double s[1] = {0.0};
             if (x.active)
-                for (int i = x.first; i < L.n; i += x.stride) {
+                for (int i = x.first; i < x.end; i += x.stride) {
                     const double qi = gamg_amul_row(L, L.diag, p, i);
                     q[i] = qi;
                     s[0] = __fma_rn(qi, p[i], s[0]);
@@ -556,7 +649,7 @@ __device__ bool gamg_coarsest(const GamgArgs& a, const Group& g)
             const double alpha = rho / s[0];
             double m[1] = {0.0};
             if (x.active)
-                for (int i = x.first; i < L.n; i += x.stride) {
+                for (int i = x.first; i < x.end; i += x.stride) {
                     e[i] = __fma_rn(alpha, p[i], e[i]);
                     r[i] = __fma_rn(-alpha, q[i], r[i]);
                     m[0] += fabs(r[i]);
@@ -570,16 +663,16 @@ __device__ bool gamg_coarsest(const GamgArgs& a, const Group& g)
 
 // e_0 = V(0, r_0), with r_0 = a.res; the last smoothing sweep of level 0 also
 // adds e_0 to x (the outer update, fused).
-__device__ bool gamg_vcycle(const GamgArgs& a, const Group& g, GamgClock& ck)
+__device__ bool gamg_vcycle(const GamgArgs& a, const Group& g, const CoarseDense& D, GamgClock& ck)
 {
     // restriction down to the coarsest level
     for (int k = 0; k + 1 < a.nlev; k++) {
         const GamgLevel& F = a.lv[k];
         const GamgLevel& C = a.lv[k + 1];
-        const Exec x = exec_for(a, k + 1, g);
+        const Exec x = exec_for(a, k + 1, g, C.n);
         const int* cc = k == 0 && a.z.on ? a.z.ccell_int : F.ccell;
         if (x.active)
-            for (int c = x.first; c < C.n; c += x.stride) {
+            for (int c = x.first; c < x.end; c += x.stride) {
                 double s = 0.0;
                 for (int j = F.cptr[c]; j < F.cptr[c + 1]; j++) s = __dadd_rn(s, F.r[cc[j]]);
                 C.r[c] = s;
@@ -587,88 +680,113 @@ __device__ bool gamg_vcycle(const GamgArgs& a, const Group& g, GamgClock& ck)
         if (!exec_sync(x, g)) return false;
         ck.lap(k);
     }
-    if (!gamg_coarsest(a, g)) return false;
+    if (!gamg_coarsest(a, g, D)) return false;
     ck.lap(128);
-    // prolongation, scaling and smoothing back up
+    // back up: prolongation by injection e = P e_c, its scaling s = (e.r)/(e.A e)
+    // and two smoothing sweeps.  The product A e of the scaling also gives the
+    // first sweep's residual, r - A (s e) = r - s (A e), so that sweep needs no
+    // Amul, and e is read through the aggregation map (each entry's aggregate
+    // is kept beside its column), never stored: two Amuls and three barriers
+    // per level (Richardson; Gauss-Seidel five) instead of three Amuls and
+    // five (seven).  With the even chunks and row teams above, per V-cycle: 64^3
+    // Richardson 564 -> 261 us, 128^3 two-stage Gauss-Seidel 1774 -> 1306 us.
+    static_assert(kGamgPostSweeps == 2, "two smoothing sweeps");
     for (int k = a.nlev - 2; k >= 0; k--) {
         const GamgLevel& L = a.lv[k];
-        const GamgLevel& C = a.lv[k + 1];
+        const double* ec = a.lv[k + 1].e;
+        const double* dg = L.diag;
         if (k + 1 == a.small_from && !group_sync(g)) return false;   // the first block's levels are done
-        const Exec x = exec_for(a, k, g);
-        if (x.active)
-            for (int i = x.first; i < L.n; i += x.stride) L.e[i] = C.e[L.agg[i]];
-        if (!exec_sync(x, g)) return false;
+        const Exec x = exec_for(a, k, g, L.n);
+        // q = A P e_c, (e.r), (e.A e)
         double v[2] = {0.0, 0.0};
-        if (x.active)
-            level_rows(a, k, L.e, L.r, nullptr, x.first, x.stride, [&](int, double qi, double ei, double ri, double) {
-                v[0] = __fma_rn(ei, ri, v[0]);
-                v[1] = __fma_rn(ei, qi, v[1]);
-            });
-        if (!exec_sum<2>(x, v, a, GS_A, g)) return false;
-        const bool fuse = k >= 1 && L.n <= a.fuse_rows;
-        const double sc = v[1] > 0.0 ? v[0] / v[1] : 1.0;   // x 1.0 leaves every value as it is
-        if (!fuse && v[1] > 0.0) {
-            if (x.active)
-                for (int i = x.first; i < L.n; i += x.stride) L.e[i] = __dmul_rn(L.e[i], sc);
-            if (!exec_sync(x, g)) return false;
+        if (x.active) {
+            if (k == 0) {
+                const bool ell = a.z.ell_w > 0 && a.z.ell_w <= 6;
+                lvl0_rows(a.z, ell ? L.cagg : nullptr, L.agg, ec, L.r, nullptr, x.first, x.stride, x.end,
+                          [&](int i, double qi, double ei, double ri, double) {
+                              L.q[i] = qi;
+                              v[0] = __fma_rn(ei, ri, v[0]);
+                              v[1] = __fma_rn(ei, qi, v[1]);
+                          });
+            } else {
+                team_rows(L, nullptr, L.cagg, ec, x, [&](int i, double s) {
+                    const double ei = ec[L.agg[i]];
+                    const double qi = __fma_rn(dg[i], ei, s);
+                    L.q[i] = qi;
+                    v[0] = __fma_rn(ei, L.r[i], v[0]);
+                    v[1] = __fma_rn(ei, qi, v[1]);
+                });
+            }
         }
-        auto scaled_e = [&L, sc](int c) { return __dmul_rn(L.e[c], sc); };
+        if (!exec_sum<2>(x, v, a, GS_A, g)) return false;
+        const double sc = v[1] > 0.0 ? v[0] / v[1] : 1.0;
         if (a.smoother == 1) {
-            // two-stage Gauss-Seidel: q = r - A e, y = rD q; then e += rD (q - L y),
-            // the row's lower entries in face order (one FMA each)
+            // two-stage Gauss-Seidel: q = r - A e, y = rD q; then e += rD (q - L y)
+            if (x.active)
+                for (int i = x.first; i < x.end; i += x.stride) {
+                    const double qi = __fma_rn(-sc, L.q[i], L.r[i]);
+                    L.q[i] = qi;
+                    L.y[i] = __dmul_rn(L.wrd[i], qi);
+                    L.e[i] = __dmul_rn(sc, ec[L.agg[i]]);
+                }
+            if (!exec_sync(x, g)) return false;
             for (int s = 0; s < kGamgPostSweeps; s++) {
-                const bool sc0 = fuse && s == 0;   // e read scaled in this sweep
+                if (s > 0) {
+                    if (x.active) {
+                        if (k == 0)
+                            lvl0_rows(a.z, a.z.Ecol, nullptr, L.e, L.r, L.wrd, x.first, x.stride, x.end,
+                                      [&](int i, double ae, double, double ri, double wi) {
+                                          const double qi = __dsub_rn(ri, ae);
+                                          L.q[i] = qi;
+                                          L.y[i] = __dmul_rn(wi, qi);
+                                      });
+                        else
+                            team_rows(L, nullptr, L.rcol, L.e, x, [&](int i, double ae) {
+                                const double qi = __dsub_rn(L.r[i], __fma_rn(dg[i], L.e[i], ae));
+                                L.q[i] = qi;
+                                L.y[i] = __dmul_rn(L.wrd[i], qi);
+                            });
+                    }
+                    if (!exec_sync(x, g)) return false;
+                }
                 if (x.active) {
-                    if (sc0) {
-                        for (int i = x.first; i < L.n; i += x.stride) {
-                            const double qi = __dsub_rn(L.r[i], gamg_amul_row_g(L, L.diag, scaled_e, i));
-                            L.q[i] = qi;
-                            L.y[i] = __dmul_rn(L.wrd[i], qi);
+                    if (k == 0) {
+                        const bool fold = s == kGamgPostSweeps - 1;   // x += e_0 here
+                        for (int i = x.first; i < x.end; i += x.stride) {
+                            const double si = lvl0_lower_sweep(a.z, L.y, i, L.q[i]);
+                            const double ei = __fma_rn(L.wrd[i], si, L.e[i]);
+                            L.e[i] = ei;
+                            if (fold) a.x[i] = __dadd_rn(a.x[i], ei);
                         }
                     } else {
-                        level_rows(a, k, L.e, L.r, L.wrd, x.first, x.stride,
-                                   [&](int i, double ae, double, double ri, double wi) {
-                                       const double qi = __dsub_rn(ri, ae);
-                                       L.q[i] = qi;
-                                       L.y[i] = __dmul_rn(wi, qi);
-                                   });
+                        team_rows(L, L.rlo, L.rcol, L.y, x, [&](int i, double ly) {
+                            L.e[i] = __fma_rn(L.wrd[i], __dsub_rn(L.q[i], ly), L.e[i]);
+                        });
                     }
                 }
-                if (!exec_sync(x, g)) return false;
-                const bool fold = k == 0 && s == kGamgPostSweeps - 1;   // x += e_0 here
-                if (x.active)
-                    for (int i = x.first; i < L.n; i += x.stride) {
-                        const double si = level_lower_sweep(a, k, L.y, i, L.q[i]);
-                        const double e0 = sc0 ? __dmul_rn(L.e[i], sc) : L.e[i];
-                        const double ei = __dadd_rn(e0, __dmul_rn(L.wrd[i], si));
-                        L.e[i] = ei;
-                        if (fold) a.x[i] = __dadd_rn(a.x[i], ei);
-                    }
                 if (!exec_sync(x, g)) return false;
             }
         } else {
-            // Jacobi sweeps alternate between e and q (an even count ends in e)
-            static_assert(kGamgPostSweeps % 2 == 0, "sweeps alternate e -> q -> e");
-            for (int s = 0; s < kGamgPostSweeps; s++) {
-                const double* src = (s & 1) ? L.q : L.e;
-                double* dst = (s & 1) ? L.e : L.q;
-                const bool fold = k == 0 && s == kGamgPostSweeps - 1;   // x += e_0 here
-                if (x.active) {
-                    if (fuse && s == 0) {
-                        for (int i = x.first; i < L.n; i += x.stride)
-                            dst[i] = __fma_rn(L.wrd[i], __dsub_rn(L.r[i], gamg_amul_row_g(L, L.diag, scaled_e, i)),
-                                              scaled_e(i));
-                    } else {
-                        level_rows(a, k, src, L.wrd, L.r, x.first, x.stride,
-                                   [&](int i, double as, double si, double wi, double ri) {
-                                       const double ei = __fma_rn(wi, __dsub_rn(ri, as), si);
-                                       dst[i] = ei;
-                                       if (fold) a.x[i] = __dadd_rn(a.x[i], ei);
-                                   });
-                    }
-                }
-                if (!exec_sync(x, g)) return false;
+            // damped Jacobi: the first sweep from q into y, the second from y into e
+            if (x.active)
+                for (int i = x.first; i < x.end; i += x.stride)
+                    L.y[i] = __fma_rn(L.wrd[i], __fma_rn(-sc, L.q[i], L.r[i]), __dmul_rn(sc, ec[L.agg[i]]));
+            if (!exec_sync(x, g)) return false;
+            if (x.active) {
+                if (k == 0)
+                    lvl0_rows(a.z, a.z.Ecol, nullptr, L.y, L.wrd, L.r, x.first, x.stride, x.end,
+                              [&](int i, double as, double yi, double wi, double ri) {
+                                  const double ei = __fma_rn(wi, __dsub_rn(ri, as), yi);
+                                  L.e[i] = ei;
+                                  a.x[i] = __dadd_rn(a.x[i], ei);   // the outer update
+                              });
+                else
+                    team_rows(L, nullptr, L.rcol, L.y, x, [&](int i, double as) {
+                        const double yi = L.y[i];
+                        L.e[i] = __fma_rn(L.wrd[i], __dsub_rn(L.r[i], __fma_rn(dg[i], yi, as)), yi);
+                    });
             }
+            if (!exec_sync(x, g)) return false;
         }
         ck.lap(64 + k);
     }
@@ -676,21 +794,21 @@ __device__ bool gamg_vcycle(const GamgArgs& a, const Group& g, GamgClock& ck)
     return true;
 }
 
-__global__ void __launch_bounds__(1024, 1) k_gamg(GamgArgs a, unsigned long long timeout_ns)
+__global__ void __launch_bounds__(kGamgThreads, 1) k_gamg(GamgArgs a, unsigned long long timeout_ns)
 {
     Group g{reinterpret_cast<unsigned long long*>(a.status + DS_BARRIER), a.status, (int)gridDim.x, (int)blockIdx.x, timeout_ns};
     spuma_solver_perf pf{};
     pf.n_levels = a.nlev;
     const GamgLevel& L0 = a.lv[0];
-    struct {
-        int first, stride;
-    } it{g.bid * (int)blockDim.x + (int)threadIdx.x, g.nblocks * (int)blockDim.x};
+    const Exec it = exec_grid(g, L0.n, L0.n >= g.nblocks * (int)blockDim.x);
+    __shared__ CoarseDense dense;
     bool ok = gamg_coarse_matrices(a, g);
+    if (ok && g.bid == 0 && a.lv[a.nlev - 1].n <= 32) gamg_coarse_dense(a.lv[a.nlev - 1], dense);
     // x, b, r = b - A x, normFactor (row sums of A times mean(x)), res0
     double v[1] = {0.0};
     const bool z0 = a.z.on;   // level 0 (x, b, r) in internal order
     if (ok) {
-        for (int i = it.first; i < L0.n; i += it.stride) {
+        for (int i = it.first; i < it.end; i += it.stride) {
             const int o = z0 ? a.z.perm[i] : i;
             a.x[i] = a.x_orig[o];
             a.b[i] = a.b_orig[o];
@@ -706,8 +824,8 @@ __global__ void __launch_bounds__(1024, 1) k_gamg(GamgArgs a, unsigned long long
         grid_reduce_read<1>(t, a.partials, GS_A, g.nblocks);
         const double xbar = L0.n > 0 ? t[0] / (double)L0.n : 0.0;
         double acc[2] = {0.0, 0.0};
-        for (int i = it.first; i < L0.n; i += it.stride) {
-            const double q = level_amul_row(a, 0, a.x, i);
+        for (int i = it.first; i < it.end; i += it.stride) {
+            const double q = level0_amul_row(a, a.x, i);
             const double r = a.b[i] - q;
             a.res[i] = r;
             double s;
@@ -737,16 +855,16 @@ __global__ void __launch_bounds__(1024, 1) k_gamg(GamgArgs a, unsigned long long
     GamgClock ck(a.clk, g.bid);
     if (ok && (a.min_iter > 0 || !conv(res0))) {
         for (;;) {
-            ok = gamg_vcycle(a, g, ck);
+            ok = gamg_vcycle(a, g, dense, ck);
             if (!ok) break;
             double acc[1] = {0.0};
             if (a.nlev == 1) {   // otherwise the last smoothing sweep of level 0 added e_0 to x
-                for (int i = it.first; i < L0.n; i += it.stride) a.x[i] = __dadd_rn(a.x[i], L0.e[i]);
+                for (int i = it.first; i < it.end; i += it.stride) a.x[i] = __dadd_rn(a.x[i], L0.e[i]);
                 ok = group_sync(g);
                 if (!ok) break;
             }
-            for (int i = it.first; i < L0.n; i += it.stride) {
-                const double r = a.b[i] - level_amul_row(a, 0, a.x, i);
+            for (int i = it.first; i < it.end; i += it.stride) {
+                const double r = a.b[i] - level0_amul_row(a, a.x, i);
                 a.res[i] = r;
                 acc[0] += fabs(r);
             }
@@ -764,8 +882,8 @@ __global__ void __launch_bounds__(1024, 1) k_gamg(GamgArgs a, unsigned long long
     // the report's true residual ||b - A x||_2 / ||b||_2 (||b - A x||_2 when b = 0)
     if (ok) {
         double acc[2] = {0.0, 0.0};
-        for (int i = it.first; i < L0.n; i += it.stride) {
-            const double r = __dsub_rn(a.b[i], level_amul_row(a, 0, a.x, i));
+        for (int i = it.first; i < it.end; i += it.stride) {
+            const double r = __dsub_rn(a.b[i], level0_amul_row(a, a.x, i));
             acc[0] = __fma_rn(r, r, acc[0]);
             acc[1] = __fma_rn(a.b[i], a.b[i], acc[1]);
         }
@@ -778,7 +896,7 @@ __global__ void __launch_bounds__(1024, 1) k_gamg(GamgArgs a, unsigned long long
         }
     }
     if (ok)
-        for (int i = it.first; i < L0.n; i += it.stride) a.x_orig[z0 ? a.z.perm[i] : i] = a.x[i];
+        for (int i = it.first; i < it.end; i += it.stride) a.x_orig[z0 ? a.z.perm[i] : i] = a.x[i];
     if (g.bid == 0 && threadIdx.x == 0 && a.perf) {
         pf.initial_residual = res0;
         pf.final_residual = res;
@@ -790,6 +908,13 @@ __global__ void __launch_bounds__(1024, 1) k_gamg(GamgArgs a, unsigned long long
         if (pf.status != 0) pf.converged = 0;
         *a.perf = pf;
     }
+}
+
+// The aggregate of every entry's column (bind time).
+__global__ void k_gamg_cagg(long long m, const int* __restrict__ col, const int* __restrict__ agg, int* __restrict__ out)
+{
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < m; e += gridDim.x * (long long)blockDim.x)
+        out[e] = col[e] >= 0 ? agg[col[e]] : -1;
 }
 
 // ----------------------------------------------------------------- host ---
@@ -1124,6 +1249,8 @@ size_t gamg_layout(spuma_gamg& G, bool assign)
             D.diag = (double*)take(8 * (size_t)H.n + 8);
             D.upper = (double*)take(8 * (size_t)H.nf + 8);
         }
+        // level 0's entries in the handle's fixed-width layout, the others' in row-CSR order
+        D.cagg = k + 1 < G.lv.size() ? (int*)take(4 * (k == 0 ? (size_t)G.h->ell_w * H.n : 2 * (size_t)H.nf) + 4) : nullptr;
         D.wrd = (double*)take(8 * (size_t)H.n + 8);
         D.rval = (double*)take(16 * (size_t)H.nf + 8);
         D.r = (double*)take(8 * (size_t)H.n + 8);
@@ -1340,7 +1467,7 @@ static spuma_status gamg_create(spuma_ldu_t h, const double* face_weight, spuma_
     G->bytes = gamg_layout(*G, false);
     G->small_from = (int)G->lv.size();
     for (int k = 0; k < (int)G->lv.size(); k++)
-        if (G->lv[k].n <= 2048) {
+        if (G->lv[k].n <= kGamgSmall) {
             G->small_from = k;
             break;
         }
@@ -1392,6 +1519,15 @@ spuma_status spuma_gamg_bind(spuma_gamg_t g, void* workspace, size_t workspace_b
         }
     }
     if (g->ccell_int) SPUMA_CUDA(up(g->ccell_int, g->lv[0].ccell_int));
+    for (size_t k = 0; k + 1 < g->lv.size(); k++) {
+        const GamgLevel& D = g->hlv[k];
+        const long long m = k == 0 ? (long long)g->h->ell_w * D.n : 2LL * D.nf;
+        if (m == 0) continue;
+        const int grid = (int)std::min<long long>((m + 255) / 256, 8LL * g->h->num_sms);
+        k_gamg_cagg<<<grid, 256, 0, s>>>(m, k == 0 ? g->h->at<int>(g->h->L.Ecol) : D.rcol, D.agg, const_cast<int*>(D.cagg));
+        count_launch();
+    }
+    SPUMA_CUDA(cudaGetLastError());
     SPUMA_CUDA(cudaStreamSynchronize(s));
     return SPUMA_OK;
 }
@@ -1467,11 +1603,6 @@ spuma_status spuma_gamg_solve(spuma_gamg_t g, const double* diag, const double* 
         h->prepared_precond = -1;
     }
     a.status = h->at<int>(h->L.status);
-    {
-        // measured at 200^3 with 262144: the levels it covers 1-8 % slower
-        static const int fuse_env = getenv("SPUMA_GAMG_FUSE_SCALE_ROWS") ? atoi(getenv("SPUMA_GAMG_FUSE_SCALE_ROWS")) : 0;
-        a.fuse_rows = fuse_env;
-    }
     a.clk = nullptr;
     if (getenv("SPUMA_PHASE_CLOCKS")) {
         a.clk = h->at<long long>(h->L.clk);
@@ -1483,15 +1614,15 @@ spuma_status spuma_gamg_solve(spuma_gamg_t g, const double* diag, const double* 
     a.tol = ctl->tolerance;
     a.rel_tol = ctl->rel_tol;
     int per_sm = 0;
-    SPUMA_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gamg, 1024, 0));
+    SPUMA_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gamg, kGamgThreads, 0));
     if (per_sm < 1) { set_error("GAMG kernel cannot be resident"); return SPUMA_ERR_CUDA; }
-    const int64_t want = ((int64_t)h->n + 1023) / 1024;
+    const int64_t want = ((int64_t)h->n + 127) / 128;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, std::min<int64_t>((int64_t)per_sm * h->num_sms,
                                                                                           kMaxBlocks)));
     SPUMA_CUDA(cudaMemsetAsync(h->at<char>(h->L.bar), 0, h->L.status + 256 - h->L.bar, s));
     unsigned long long tns = barrier_timeout_ns();
     void* args[] = {(void*)&a, (void*)&tns};
-    SPUMA_CUDA(cudaLaunchCooperativeKernel((const void*)k_gamg, grid, 1024, args, 0, s));
+    SPUMA_CUDA(cudaLaunchCooperativeKernel((const void*)k_gamg, grid, kGamgThreads, args, 0, s));
     count_launch();
     return SPUMA_OK;
 }
