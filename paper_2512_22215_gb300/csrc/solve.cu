@@ -614,17 +614,12 @@ __device__ bool phase_factor(const SolveArgs& a, const Group& g)
 }
 
 // ------------------------------------------------------ DIC sweeps ---------
-// What the sweeps' reduction takes: rho = w.r (PCG), rho = w.dotv with a
-// vector of the caller's (PBiCG: wA.rT), or nothing (PBiCG's M^-T apply).
-// A template argument, so that the PCG kernels keep their own code.
-enum RhoWith { RHO_R = 0, RHO_VEC = 1, RHO_NONE = 2 };
-
 // Forward rows of one level: w = rD r - sum (rD a) w_lower (ascending face
 // order); with `rho` (top level: no upper neighbours, so w is final here)
-// also rho += w r (or w dotv).
-template <class T, int RW>
+// also rho += w r.
+template <class T>
 __device__ __forceinline__ void fwd_rows(const Mat<T>& A, Vecs<T> v, int r0, int r1, int first, int stride, bool rho,
-                                         const T* dotv, Acc<T>& arho)
+                                         Acc<T>& arho)
 {
     constexpr int R = ChainShape<T>::R, G = ChainShape<T>::G;
     for (int pb = r0 + first; pb < r1; pb += R * stride) {
@@ -645,16 +640,16 @@ __device__ __forceinline__ void fwd_rows(const Mat<T>& A, Vecs<T> v, int r0, int
         for (int k = 0; k < R; k++)
             if (ok[k]) {
                 v.w[p[k]] = ww[k];
-                if (RW != RHO_NONE && rho) arho.prod(ww[k], RW == RHO_R ? rr[k] : dotv[p[k]]);
+                if (rho) arho.prod(ww[k], rr[k]);
             }
     }
 }
 
 // Backward rows of one level: w -= sum (rD a) w_upper (descending face
-// order); rho += w r (or w dotv).
-template <class T, int RW>
+// order); rho += w r.
+template <class T>
 __device__ __forceinline__ void bwd_rows(const Mat<T>& A, Vecs<T> v, int r0, int r1, int first, int stride,
-                                         const T* dotv, Acc<T>& arho)
+                                         Acc<T>& arho)
 {
     constexpr int R = ChainShape<T>::R, G = ChainShape<T>::G;
     // row extents one round ahead: the next round's are loaded while this
@@ -688,7 +683,7 @@ __device__ __forceinline__ void bwd_rows(const Mat<T>& A, Vecs<T> v, int r0, int
         for (int k = 0; k < R; k++)
             if (ok[k]) {
                 v.w[p[k]] = ww[k];
-                if (RW != RHO_NONE) arho.prod(ww[k], RW == RHO_R ? v.r[p[k]] : dotv[p[k]]);
+                arho.prod(ww[k], v.r[p[k]]);
             }
     }
 }
@@ -705,7 +700,7 @@ __device__ __forceinline__ void level_chunk(const int* lvl, int L, int nblocks, 
 }
 
 // w = M^-1 r with the DIC (or DILU) factor held in A's sweep coefficients,
-// and the block partials of rho (RhoWith) in `slot` before the last grid
+// and the block partials of rho = w.r in SL_B before the last grid
 // barrier.  Forward sweep over levels 0 .. nlev-1, backward over nlev-2 .. 0
 // (the top level has no upper neighbours: its backward step would leave w
 // as it is, so its rho terms are taken in the forward step), one grid
@@ -716,18 +711,17 @@ __device__ __forceinline__ void level_chunk(const int* lvl, int L, int nblocks, 
 // of every level (the same 1/nblocks share of each level's Morton order);
 // 0, a level's rows strided over the group in blockDim-row pieces.  Measured
 // at 200^3: mixed solve 328.8 against 333.5 ms, FP64 582.5 against 599.7 ms.
-template <class T, int RW = RHO_R>
-__device__ bool dic_apply(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, const Group& g, PhaseClock& pc,
-                          const T* dotv = nullptr, int slot = SL_B)
+template <class T>
+__device__ bool dic_apply(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, const Group& g, PhaseClock& pc)
 {
     const RowIter it = rows_of(g);
     const int nlev = a.nlev, tail = min(a.tail_from, nlev);
     const int tid = (int)threadIdx.x, bs = (int)blockDim.x;
     Acc<T> arho;
     auto end_step = [&](bool last) {
-        if (RW != RHO_NONE && last) {
+        if (last) {
             double t[1] = {arho.value()};
-            block_reduce_store<1>(t, a.partials, slot, g.bid);
+            block_reduce_store<1>(t, a.partials, SL_B, g.bid);
         }
         return group_sync(g);
     };
@@ -748,18 +742,18 @@ __device__ bool dic_apply(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, const 
     for (int L = 0; L < tail; L++) {
         int c0, c1, first, stride;
         rows(L, c0, c1, first, stride);
-        fwd_rows<T, RW>(A, v, c0, c1, first, stride, L == nlev - 1, dotv, arho);
+        fwd_rows<T>(A, v, c0, c1, first, stride, L == nlev - 1, arho);
         if (!end_step(nlev == 1)) return false;
         pc.lap(CK_FWD + min(L, 63));
     }
     if (tail < nlev) {
         if (g.bid == 0) {
             for (int L = tail; L < nlev; L++) {
-                fwd_rows<T, RW>(A, v, a.lvl[L], a.lvl[L + 1], tid, bs, L == nlev - 1, dotv, arho);
+                fwd_rows<T>(A, v, a.lvl[L], a.lvl[L + 1], tid, bs, L == nlev - 1, arho);
                 __syncthreads();
             }
             for (int L = nlev - 2; L >= tail; L--) {
-                bwd_rows<T, RW>(A, v, a.lvl[L], a.lvl[L + 1], tid, bs, dotv, arho);
+                bwd_rows<T>(A, v, a.lvl[L], a.lvl[L + 1], tid, bs, arho);
                 __syncthreads();
             }
         }
@@ -769,7 +763,7 @@ __device__ bool dic_apply(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, const 
     for (int L = min(tail, nlev - 1) - 1; L >= 0; L--) {
         int c0, c1, first, stride;
         rows(L, c0, c1, first, stride);
-        bwd_rows<T, RW>(A, v, c0, c1, first, stride, dotv, arho);
+        bwd_rows<T>(A, v, c0, c1, first, stride, arho);
         if (!end_step(L == 0)) return false;
         pc.lap(CK_BWD + min(L, 63));
     }
@@ -1247,6 +1241,126 @@ __device__ bool solve_mixed_restart(const SolveArgs& a, const Group& g, double n
 // Kinds of persistent launch, one kernel each so that every kernel holds only
 // its own path (register allocation is per kernel).
 // -------------------------------------------------------------- PBiCG ---
+// One level's rows of both DILU applies (A and A^T) in one direction: they
+// share the level's structure, so the extents and columns are read once, and
+// the two chains' gathers are in flight together.  FWD: w = rD r - sum c w_l,
+// else w -= sum c w_u (descending) and rho += wA rT.
+template <bool FWD, int G>
+__device__ __forceinline__ void dilu_rows(const Mat<double>& A, const Mat<double>& AT, const double* rA,
+                                          const double* rT, double* wA, double* wT, int r0, int r1, int first,
+                                          int stride, bool rho, Acc<double>& arho)
+{
+    const int* ptr = FWD ? A.Lptr : A.Uptr;
+    const int* col = FWD ? A.Lcol : A.Ucol;
+    const double *ca = FWD ? A.Lc : A.Uc, *ct = FWD ? AT.Lc : AT.Uc;
+    int p = r0 + first;
+    int n0 = p < r1 ? __ldcs(ptr + p) : 0, n1 = p < r1 ? __ldcs(ptr + p + 1) : 0;
+    for (; p < r1; p += stride) {
+        const int e0 = n0, e1 = n1, pn = p + stride;
+        n0 = pn < r1 ? __ldcs(ptr + pn) : 0;
+        n1 = pn < r1 ? __ldcs(ptr + pn + 1) : 0;
+        const double rt = rT[p];
+        double ya, yt;
+        if (FWD) {
+            const double rd = __ldcs(A.rD + p);
+            ya = mul_rn(rd, rA[p]);
+            yt = mul_rn(rd, rt);
+        } else {
+            ya = wA[p];
+            yt = wT[p];
+        }
+        for (int off = 0; off < e1 - e0; off += G) {
+            int c[G];
+            double a[G], t[G], xa[G], xt[G];
+#pragma unroll
+            for (int j = 0; j < G; j++) {
+                const int e = FWD ? e0 + off + j : e1 - 1 - off - j;
+                const bool ok = FWD ? e < e1 : e >= e0;
+                c[j] = ok ? __ldcs(col + e) : -1;
+                a[j] = ok ? __ldcs(ca + e) : 0.0;
+                t[j] = ok ? __ldcs(ct + e) : 0.0;
+            }
+#pragma unroll
+            for (int j = 0; j < G; j++) {
+                xa[j] = c[j] >= 0 ? wA[c[j]] : 0.0;
+                xt[j] = c[j] >= 0 ? wT[c[j]] : 0.0;
+            }
+#pragma unroll
+            for (int j = 0; j < G; j++)
+                if (c[j] >= 0) {
+                    ya = fmadd(-a[j], xa[j], ya);
+                    yt = fmadd(-t[j], xt[j], yt);
+                }
+        }
+        wA[p] = ya;
+        wT[p] = yt;
+        if (rho) arho.prod(ya, rt);
+    }
+}
+
+// wA = M^-1 rA and wT = M^-T rT, level by level together (as dic_apply: one
+// grid barrier per level, the small last levels on the first block alone),
+// with the partials of rho = wA.rT in SL_B before the last barrier.  The two
+// applies one after the other took twice the barriers and read the extents
+// and columns twice: 128^3, DILU, an iteration 517 -> 381 us.
+__device__ bool dilu_apply(const SolveArgs& a, const Mat<double>& A, const Mat<double>& AT, const double* rA,
+                           const double* rT, double* wA, double* wT, const Group& g, PhaseClock& pc)
+{
+    constexpr int G = 3;
+    const RowIter it = rows_of(g);
+    const int nlev = a.nlev, tail = min(a.tail_from, nlev);
+    const int tid = (int)threadIdx.x, bs = (int)blockDim.x;
+    Acc<double> arho;
+    auto end_step = [&](bool last) {
+        if (last) {
+            double t[1] = {arho.value()};
+            block_reduce_store<1>(t, a.partials, SL_B, g.bid);
+        }
+        return group_sync(g);
+    };
+    if (nlev == 0) return end_step(true);
+    auto rows = [&](int L, int& c0, int& c1, int& first, int& stride) {
+        if (a.sweep != 0) {
+            level_chunk(a.lvl, L, g.nblocks, g.bid, c0, c1);
+            first = tid;
+            stride = bs;
+        } else {
+            c0 = a.lvl[L];
+            c1 = a.lvl[L + 1];
+            first = it.first;
+            stride = it.stride;
+        }
+    };
+    int c0, c1, first, stride;
+    for (int L = 0; L < tail; L++) {
+        rows(L, c0, c1, first, stride);
+        dilu_rows<true, G>(A, AT, rA, rT, wA, wT, c0, c1, first, stride, L == nlev - 1, arho);
+        if (!end_step(nlev == 1)) return false;
+        pc.lap(CK_FWD + min(L, 63));
+    }
+    if (tail < nlev) {
+        if (g.bid == 0) {
+            for (int L = tail; L < nlev; L++) {
+                dilu_rows<true, G>(A, AT, rA, rT, wA, wT, a.lvl[L], a.lvl[L + 1], tid, bs, L == nlev - 1, arho);
+                __syncthreads();
+            }
+            for (int L = nlev - 2; L >= tail; L--) {
+                dilu_rows<false, G>(A, AT, rA, rT, wA, wT, a.lvl[L], a.lvl[L + 1], tid, bs, true, arho);
+                __syncthreads();
+            }
+        }
+        if (!end_step(tail == 0)) return false;
+        pc.lap(CK_FWD + min(tail, 63));
+    }
+    for (int L = min(tail, nlev - 1) - 1; L >= 0; L--) {
+        rows(L, c0, c1, first, stride);
+        dilu_rows<false, G>(A, AT, rA, rT, wA, wT, c0, c1, first, stride, true, arho);
+        if (!end_step(L == 0)) return false;
+        pc.lap(CK_BWD + min(L, 63));
+    }
+    return true;
+}
+
 // OpenFOAM PBiCG on an asymmetric matrix (the paper's momentum solver: PBiCG
 // with DILU), FP64, after phase_init (x, rA = b - A x, normFactor from the
 // row sums of A).  Vectors: x, rA = r, wA = w, pA = p, wT = q, rT = b (the
@@ -1265,6 +1379,8 @@ __device__ bool solve_pbicg(const SolveArgs& a, const Group& g, double nfac, dou
     AT.Ea = a.EaT64;
     double *x = a.x, *rA = a.r, *wA = a.w, *pA = a.p, *wT = a.q, *rT = a.b, *pT = a.pT;
     PhaseClock pc(a.phase_clk, g.bid);
+    const int nv = a.n / 2;   // 16-byte pairs of the streaming passes
+    auto d2 = [](double* q) { return reinterpret_cast<double2*>(q); };
     for (int p = it.first; p < a.n; p += it.stride) rT[p] = a.b[p] - amul_row<double>(AT, x, p);
     if (!group_sync(g)) return false;
     double res = res0;
@@ -1275,7 +1391,15 @@ __device__ bool solve_pbicg(const SolveArgs& a, const Group& g, double nfac, dou
         for (;;) {
             if (pending) {
                 double acc[1] = {0.0};
-                for (int p = it.first; p < a.n; p += it.stride) {
+                for (int i = it.first; i < nv; i += it.stride) {
+                    const double2 ra = vfma(-alpha, d2(wA)[i], d2(rA)[i]), rt = vfma(-alpha, d2(wT)[i], d2(rT)[i]);
+                    __stcs(d2(x) + i, vfma(alpha, d2(pA)[i], __ldcs(d2(x) + i)));
+                    d2(rA)[i] = ra;
+                    d2(rT)[i] = rt;
+                    acc[0] += fabs(ra.x);
+                    acc[0] += fabs(ra.y);
+                }
+                for (int p = 2 * nv + it.first; p < a.n; p += it.stride) {
                     x[p] = fmadd(alpha, pA[p], x[p]);
                     rA[p] = fmadd(-alpha, wA[p], rA[p]);
                     rT[p] = fmadd(-alpha, wT[p], rT[p]);
@@ -1291,8 +1415,7 @@ __device__ bool solve_pbicg(const SolveArgs& a, const Group& g, double nfac, dou
             }
             wArA_old = wArA;
             if (a.precond == SPUMA_PRECOND_DILU) {
-                if (!dic_apply<double, RHO_VEC>(a, A, Vecs<double>{x, rA, wA, pA, wT}, g, pc, rT, SL_B)) return false;
-                if (!dic_apply<double, RHO_NONE>(a, AT, Vecs<double>{x, rT, wT, pT, wA}, g, pc)) return false;
+                if (!dilu_apply(a, A, AT, rA, rT, wA, wT, g, pc)) return false;
             } else {
                 double acc[1] = {0.0};
                 for (int p = it.first; p < a.n; p += it.stride) {
@@ -1310,7 +1433,12 @@ __device__ bool solve_pbicg(const SolveArgs& a, const Group& g, double nfac, dou
             wArA = t[0];
             const bool first = !pending;
             const double beta = first ? 0.0 : wArA / wArA_old;
-            for (int p = it.first; p < a.n; p += it.stride) {
+            for (int i = it.first; i < nv; i += it.stride) {
+                const double2 wa = d2(wA)[i], wt = d2(wT)[i];
+                d2(pA)[i] = first ? wa : vfma(beta, d2(pA)[i], wa);
+                d2(pT)[i] = first ? wt : vfma(beta, d2(pT)[i], wt);
+            }
+            for (int p = 2 * nv + it.first; p < a.n; p += it.stride) {
                 pA[p] = first ? wA[p] : fmadd(beta, pA[p], wA[p]);
                 pT[p] = first ? wT[p] : fmadd(beta, pT[p], wT[p]);
             }
