@@ -120,6 +120,12 @@ struct Group {
     int nblocks;           // blocks in the group
     int bid;               // this block's index in the group
     unsigned long long timeout_ns;
+    static constexpr bool wide = false;
+};
+// A group of blocks of at most 512 threads, whose kernels have 128 registers
+// per thread: their solver phases keep one round of loads ahead.
+struct WideGroup : Group {
+    static constexpr bool wide = true;
 };
 
 // Returns true when the caller may continue (no error recorded anywhere).

@@ -699,6 +699,184 @@ __device__ __forceinline__ void level_chunk(const int* lvl, int L, int nblocks, 
     c1 = min(c0 + chunk, r1);
 }
 
+// This block's chunks of the first kChunkTable levels, in shared memory, filled
+// once per launch (fill_chunk_table) for the wide sweeps.
+constexpr int kChunkTable = 256;
+__device__ __forceinline__ int2* chunk_table()
+{
+    __shared__ int2 table[kChunkTable];
+    return table;
+}
+__device__ __forceinline__ void fill_chunk_table(const SolveArgs& a, const Group& g)
+{
+    int2* t = chunk_table();
+    for (int L = threadIdx.x; L < min(a.nlev, kChunkTable); L += blockDim.x) {
+        int c0, c1;
+        level_chunk(a.lvl, L, g.nblocks, g.bid, c0, c1);
+        t[L] = make_int2(c0, c1);
+    }
+    __syncthreads();
+}
+
+// The sweeps with 128 registers per thread (WideGroup).  A level's row takes
+// three dependent memory round trips (extents; columns and coefficients;
+// gathers of w), and only the last depends on the previous level: so a
+// thread's rounds, taken over all its levels as one sequence, are pipelined
+// across the grid barriers, the extents two rounds ahead and the entries, r and
+// rD (or the row's own w) one round ahead.  After a barrier only the gathers,
+// the FMA chain and the store remain.  Warp 0 takes no rows: its first thread
+// is the one that arrives at the grid barrier, and the fence of that arrival
+// would wait for the warp's own loads ahead.
+template <class T>
+struct WideShape {
+    static constexpr int R = sizeof(T) == 4 ? 2 : 1;   // rows per thread and round
+    static constexpr int G = 6;
+};
+
+// The thread's rounds: row pb (and pb + stride ...) of level L, below c1.
+struct RoundIter {
+    int L, pb, c1;
+};
+
+template <class T, int R, int G>
+struct SweepRound {
+    int e0[R], e1[R], c[R][G];
+    T cf[R][G], rr[R], ww[R];
+};
+
+// FWD: levels from .. to-1 ascending, else to-1 .. from descending.  SOLO: the
+// calling block takes whole levels by itself, with block barriers between them.
+template <class T, bool FWD, bool SOLO, class GR>
+__device__ __forceinline__ bool wide_sweep(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, const GR& g, PhaseClock& pc,
+                                           int from, int to, Acc<T>& arho, bool rho_last)
+{
+    constexpr int R = WideShape<T>::R, G = WideShape<T>::G;
+    // blocks of one warp keep it at work
+    const int service = !SOLO && blockDim.x > kWarp ? kWarp : 0;
+    const int nlev = a.nlev, tid = (int)threadIdx.x - service, bs = (int)blockDim.x - service;
+    const bool chunks = !SOLO && a.sweep != 0, own = SOLO || chunks;
+    const int first = own ? tid : g.bid * bs + tid, stride = own ? bs : g.nblocks * bs;
+    const int2* table = chunk_table();
+    const int* ptr = FWD ? A.Lptr : A.Uptr;
+    const int* col = FWD ? A.Lcol : A.Ucol;
+    const T* coef = FWD ? A.Lc : A.Uc;
+    const unsigned long long pol = keep_policy<T, true>();
+    const int Lbeg = FWD ? from : to - 1, Lend = FWD ? to : from - 1;
+    auto open = [&](RoundIter& it) {   // first round of level it.L, or of the next level that has one
+        if (tid < 0) it.L = Lend;
+        while (it.L != Lend) {
+            int c0;
+            if (chunks && it.L < kChunkTable) {
+                c0 = table[it.L].x;
+                it.c1 = table[it.L].y;
+            } else if (chunks) {
+                level_chunk(a.lvl, it.L, g.nblocks, g.bid, c0, it.c1);
+            } else {
+                c0 = a.lvl[it.L];
+                it.c1 = a.lvl[it.L + 1];
+            }
+            it.pb = c0 + first;
+            if (it.pb < it.c1) return;
+            it.L += FWD ? 1 : -1;
+        }
+    };
+    auto next = [&](RoundIter& it) {
+        it.pb += R * stride;
+        if (it.pb < it.c1) return;
+        it.L += FWD ? 1 : -1;
+        open(it);
+    };
+    auto extents = [&](const RoundIter& it, int (&e0)[R], int (&e1)[R]) {
+#pragma unroll
+        for (int k = 0; k < R; k++) {
+            const int p = it.pb + k * stride;
+            const bool ok = it.L != Lend && p < it.c1;
+            e0[k] = ok ? __ldcs(ptr + p) : 0;
+            e1[k] = ok ? __ldcs(ptr + p + 1) : 0;
+        }
+    };
+    auto entries = [&](const RoundIter& it, SweepRound<T, R, G>& q) {
+#pragma unroll
+        for (int k = 0; k < R; k++) {
+            const int p = it.pb + k * stride;
+            const bool ok = it.L != Lend && p < it.c1;
+            if (FWD) {
+                q.rr[k] = ok ? v.r[p] : T(0);
+                q.ww[k] = ok ? __ldcs(A.rD + p) : T(0);
+            } else {
+                q.ww[k] = ok ? v.w[p] : T(0);
+                q.rr[k] = ok ? v.r[p] : T(0);
+            }
+#pragma unroll
+            for (int j = 0; j < G; j++) {
+                const int e = FWD ? q.e0[k] + j : q.e1[k] - 1 - j;
+                const bool has = FWD ? e < q.e1[k] : e >= q.e0[k];
+                q.c[k][j] = has ? __ldcs(col + e) : -1;
+                q.cf[k][j] = has ? __ldcs(coef + e) : T(0);
+            }
+        }
+    };
+    RoundIter cur{Lbeg, 0, 0}, nxt, nn;
+    SweepRound<T, R, G> q, qn;
+    int n0[R], n1[R];
+    open(cur);
+    nxt = cur;
+    if (nxt.L != Lend) next(nxt);
+    extents(cur, q.e0, q.e1);
+    extents(nxt, n0, n1);
+    entries(cur, q);
+    for (int L = Lbeg; L != Lend; L += FWD ? 1 : -1) {
+        while (cur.L == L) {
+            // this round's gathers, then the entries of the next round and the
+            // extents of the one after
+            T x[R][G], acc[R];
+#pragma unroll
+            for (int k = 0; k < R; k++)
+#pragma unroll
+                for (int j = 0; j < G; j++) x[k][j] = q.c[k][j] >= 0 ? gather<true>(v.w, q.c[k][j], pol) : T(0);
+#pragma unroll
+            for (int k = 0; k < R; k++) {
+                qn.e0[k] = n0[k];
+                qn.e1[k] = n1[k];
+            }
+            entries(nxt, qn);
+            nn = nxt;
+            if (nn.L != Lend) next(nn);
+            extents(nn, n0, n1);
+#pragma unroll
+            for (int k = 0; k < R; k++) {
+                acc[k] = FWD ? mul_rn(q.ww[k], q.rr[k]) : q.ww[k];
+#pragma unroll
+                for (int j = 0; j < G; j++)
+                    if (q.c[k][j] >= 0) acc[k] = fmadd(-q.cf[k][j], x[k][j], acc[k]);
+                for (int j = G; j < q.e1[k] - q.e0[k]; j++) {   // rows of more than G entries
+                    const int e = FWD ? q.e0[k] + j : q.e1[k] - 1 - j;
+                    acc[k] = fmadd(-__ldcs(coef + e), v.w[__ldcs(col + e)], acc[k]);
+                }
+                const int p = cur.pb + k * stride;
+                if (p < cur.c1) {
+                    v.w[p] = acc[k];
+                    if (!FWD || L == nlev - 1) arho.prod(acc[k], q.rr[k]);   // top level: w is final here
+                }
+            }
+            cur = nxt;
+            q = qn;
+            nxt = nn;
+        }
+        if (SOLO) {
+            __syncthreads();
+            continue;
+        }
+        if (rho_last && (FWD ? L == nlev - 1 : L == 0)) {
+            double t[1] = {arho.value()};
+            block_reduce_store<1>(t, a.partials, SL_B, g.bid);
+        }
+        if (!group_sync(g)) return false;
+        pc.lap((FWD ? CK_FWD : CK_BWD) + min(L, 63));
+    }
+    return true;
+}
+
 // w = M^-1 r with the DIC (or DILU) factor held in A's sweep coefficients,
 // and the block partials of rho = w.r in SL_B before the last grid
 // barrier.  Forward sweep over levels 0 .. nlev-1, backward over nlev-2 .. 0
@@ -711,8 +889,8 @@ __device__ __forceinline__ void level_chunk(const int* lvl, int L, int nblocks, 
 // of every level (the same 1/nblocks share of each level's Morton order);
 // 0, a level's rows strided over the group in blockDim-row pieces.  Measured
 // at 200^3: mixed solve 328.8 against 333.5 ms, FP64 582.5 against 599.7 ms.
-template <class T>
-__device__ bool dic_apply(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, const Group& g, PhaseClock& pc)
+template <class T, class GR>
+__device__ bool dic_apply(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, const GR& g, PhaseClock& pc)
 {
     const RowIter it = rows_of(g);
     const int nlev = a.nlev, tail = min(a.tail_from, nlev);
@@ -739,33 +917,46 @@ __device__ bool dic_apply(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, const 
             stride = it.stride;
         }
     };
-    for (int L = 0; L < tail; L++) {
-        int c0, c1, first, stride;
-        rows(L, c0, c1, first, stride);
-        fwd_rows<T>(A, v, c0, c1, first, stride, L == nlev - 1, arho);
-        if (!end_step(nlev == 1)) return false;
-        pc.lap(CK_FWD + min(L, 63));
+    if constexpr (GR::wide) {
+        if (!wide_sweep<T, true, false>(a, A, v, g, pc, 0, tail, arho, nlev == 1)) return false;
+    } else {
+        for (int L = 0; L < tail; L++) {
+            int c0, c1, first, stride;
+            rows(L, c0, c1, first, stride);
+            fwd_rows<T>(A, v, c0, c1, first, stride, L == nlev - 1, arho);
+            if (!end_step(nlev == 1)) return false;
+            pc.lap(CK_FWD + min(L, 63));
+        }
     }
     if (tail < nlev) {
         if (g.bid == 0) {
-            for (int L = tail; L < nlev; L++) {
-                fwd_rows<T>(A, v, a.lvl[L], a.lvl[L + 1], tid, bs, L == nlev - 1, arho);
-                __syncthreads();
-            }
-            for (int L = nlev - 2; L >= tail; L--) {
-                bwd_rows<T>(A, v, a.lvl[L], a.lvl[L + 1], tid, bs, arho);
-                __syncthreads();
+            if constexpr (GR::wide) {
+                wide_sweep<T, true, true>(a, A, v, g, pc, tail, nlev, arho, false);
+                wide_sweep<T, false, true>(a, A, v, g, pc, tail, nlev - 1, arho, false);
+            } else {
+                for (int L = tail; L < nlev; L++) {
+                    fwd_rows<T>(A, v, a.lvl[L], a.lvl[L + 1], tid, bs, L == nlev - 1, arho);
+                    __syncthreads();
+                }
+                for (int L = nlev - 2; L >= tail; L--) {
+                    bwd_rows<T>(A, v, a.lvl[L], a.lvl[L + 1], tid, bs, arho);
+                    __syncthreads();
+                }
             }
         }
         if (!end_step(tail == 0)) return false;
         pc.lap(CK_FWD + min(tail, 63));
     }
-    for (int L = min(tail, nlev - 1) - 1; L >= 0; L--) {
-        int c0, c1, first, stride;
-        rows(L, c0, c1, first, stride);
-        bwd_rows<T>(A, v, c0, c1, first, stride, arho);
-        if (!end_step(L == 0)) return false;
-        pc.lap(CK_BWD + min(L, 63));
+    if constexpr (GR::wide) {
+        return wide_sweep<T, false, false>(a, A, v, g, pc, 0, min(tail, nlev - 1), arho, true);
+    } else {
+        for (int L = min(tail, nlev - 1) - 1; L >= 0; L--) {
+            int c0, c1, first, stride;
+            rows(L, c0, c1, first, stride);
+            bwd_rows<T>(A, v, c0, c1, first, stride, arho);
+            if (!end_step(L == 0)) return false;
+            pc.lap(CK_BWD + min(L, 63));
+        }
     }
     return true;
 }
@@ -826,8 +1017,8 @@ __device__ bool diag_pass(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, bool p
 }
 
 // p = w (first) or w + beta p; 16-byte loads, scalar tail
-template <class T>
-__device__ bool search_direction(const SolveArgs& a, Vecs<T> v, bool first, T beta, const Group& g)
+template <class T, class GR>
+__device__ bool search_direction(const SolveArgs& a, Vecs<T> v, bool first, T beta, const GR& g)
 {
     using VT = typename V16<T>::type;
     constexpr int W = V16<T>::n;
@@ -835,7 +1026,22 @@ __device__ bool search_direction(const SolveArgs& a, Vecs<T> v, bool first, T be
     const int nv = a.n / W;
     VT* pv = reinterpret_cast<VT*>(v.p);
     const VT* wv = reinterpret_cast<const VT*>(v.w);
-    for (int i = it.first; i < nv; i += it.stride) {
+    int i = it.first;
+    if constexpr (GR::wide) {   // two at a time: half the threads, as many bytes in flight
+        for (; i + it.stride < nv; i += 2 * it.stride) {
+            const VT w0 = wv[i], w1 = wv[i + it.stride];
+            VT p0 = w0, p1 = w1;
+            if (!first) {
+                p0 = pv[i];
+                p1 = pv[i + it.stride];
+                p0 = vfma(beta, p0, w0);
+                p1 = vfma(beta, p1, w1);
+            }
+            pv[i] = p0;
+            pv[i + it.stride] = p1;
+        }
+    }
+    for (; i < nv; i += it.stride) {
         const VT ww = wv[i];
         pv[i] = first ? ww : vfma(beta, pv[i], ww);
     }
@@ -844,16 +1050,16 @@ __device__ bool search_direction(const SolveArgs& a, Vecs<T> v, bool first, T be
 }
 
 // q = A p and sigma = q.p
-template <class T>
-__device__ bool amul_sigma(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, const Group& g, double* sigma)
+template <class T, class GR>
+__device__ bool amul_sigma(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, const GR& g, double* sigma)
 {
     constexpr int R = AmulShape<T>::R, G = AmulShape<T>::G;
     Acc<T> asig;
     RowIter it = rows_of(g);
     // rows [r0, r1) from `first` with `stride`
     auto range = [&](int r0, int r1, int first, int stride) {
-        if (PipeShape<T>::in_solver && A.ell_w > 0 && A.ell_w <= PipeShape<T>::G) {
-            ell_amul_pipelined<T, PipeShape<T>::R, PipeShape<T>::G>(A, v.p, r0 + first, stride, r1,
+        if ((PipeShape<T>::in_solver || GR::wide) && A.ell_w > 0 && A.ell_w <= PipeShape<T>::G) {
+            ell_amul_pipelined<T, GR::wide ? 2 : PipeShape<T>::R, PipeShape<T>::G>(A, v.p, r0 + first, stride, r1,
                                                                     [&](int p, T y, T xp) {
                                                                         v.q[p] = y;
                                                                         asig.prod(y, xp);
@@ -899,8 +1105,8 @@ __device__ bool amul_sigma(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, const
 
 // x += alpha p, r -= alpha q and sum|r| as a pass of its own, ahead of the
 // forward sweep (16-byte loads, scalar tail).
-template <class T>
-__device__ bool update_pass(const SolveArgs& a, Vecs<T> v, T alpha, const Group& g, double* ressum)
+template <class T, class GR>
+__device__ bool update_pass(const SolveArgs& a, Vecs<T> v, T alpha, const GR& g, double* ressum)
 {
     using VT = typename V16<T>::type;
     constexpr int W = V16<T>::n;
@@ -911,7 +1117,22 @@ __device__ bool update_pass(const SolveArgs& a, Vecs<T> v, T alpha, const Group&
     VT* rv = reinterpret_cast<VT*>(v.r);
     const VT* pv = reinterpret_cast<const VT*>(v.p);
     const VT* qv = reinterpret_cast<const VT*>(v.q);
-    for (int i = it.first; i < nv; i += it.stride) {
+    int i = it.first;
+    if constexpr (GR::wide) {
+        for (; i + it.stride < nv; i += 2 * it.stride) {
+            const int i2 = i + it.stride;
+            const VT q0 = qv[i], q1 = qv[i2], r0 = rv[i], r1 = rv[i2], p0 = pv[i], p1 = pv[i2];
+            const VT x0 = __ldcs(xv + i), x1 = __ldcs(xv + i2);
+            const VT s0 = vfma(-alpha, q0, r0), s1 = vfma(-alpha, q1, r1);
+            __stcs(xv + i, vfma(alpha, p0, x0));
+            __stcs(xv + i2, vfma(alpha, p1, x1));
+            rv[i] = s0;
+            rv[i2] = s1;
+            vadd_abs(acc, s0);
+            vadd_abs(acc, s1);
+        }
+    }
+    for (; i < nv; i += it.stride) {
         const VT rr = vfma(-alpha, qv[i], rv[i]);
         __stcs(xv + i, vfma(alpha, pv[i], __ldcs(xv + i)));
         rv[i] = rr;
@@ -937,8 +1158,8 @@ __device__ bool update_pass(const SolveArgs& a, Vecs<T> v, T alpha, const Group&
 // (1), lets it go on (0) or replaces r and asks for w to be computed from the
 // new r (2).
 // Returns 0 (w and rho ready), 2 (stop) or -1 (device error).
-template <class T, class AfterUpdate>
-__device__ int precondition(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, bool pending, T alpha, const Group& g,
+template <class T, class AfterUpdate, class GR>
+__device__ int precondition(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, bool pending, T alpha, const GR& g,
                             PhaseClock& pc, double* rho, AfterUpdate after_update)
 {
     if (a.precond == SPUMA_PRECOND_DIC) {
@@ -969,10 +1190,10 @@ __device__ int precondition(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, bool
 
 // PCG iterations on (A, v.r) from the current v.x (OpenFOAM recurrences).
 // Returns the iteration count, or -1 when a device error stopped the group.
-template <class T>
+template <class T, class GR>
 __device__ int pcg_loop(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, double nfac, double res0, double tol,
                         double rel_tol, int max_iter, int min_iter, double* res_out, int* singular,
-                        const Group& g)
+                        const GR& g)
 {
     PhaseClock pc(a.phase_clk, g.bid);
     double res = res0;
@@ -1046,7 +1267,8 @@ __device__ bool refine_residual(const SolveArgs& a, const Group& g, bool fold, d
 // FP32 residual has dropped by inner_rel_tol since the last replacement, the
 // FP32 residual claims convergence, or max_iter is reached; the search
 // direction is kept, so the Krylov space is never restarted.
-__device__ bool solve_mixed_reliable(const SolveArgs& a, const Group& g, double nfac, double res0,
+template <class GR>
+__device__ bool solve_mixed_reliable(const SolveArgs& a, const GR& g, double nfac, double res0,
                                      spuma_solver_perf& pf)
 {
     RowIter it = rows_of(g);
@@ -1190,7 +1412,8 @@ __device__ void phase_store_x(const SolveArgs& a, const Group& g)
 
 // Mixed precision, restarted form: FP64 refinement around FP32 inner PCG
 // solves of A d = r / max|r| from d = 0 to inner_rel_tol.
-__device__ bool solve_mixed_restart(const SolveArgs& a, const Group& g, double nfac, spuma_solver_perf& pf)
+template <class GR>
+__device__ bool solve_mixed_restart(const SolveArgs& a, const GR& g, double nfac, spuma_solver_perf& pf)
 {
     RowIter it = rows_of(g);
     const Mat<float> A32 = mat_of<float>(a);
@@ -1303,10 +1526,11 @@ __device__ __forceinline__ void dilu_rows(const Mat<double>& A, const Mat<double
 // with the partials of rho = wA.rT in SL_B before the last barrier.  The two
 // applies one after the other took twice the barriers and read the extents
 // and columns twice: 128^3, DILU, an iteration 517 -> 381 us.
+template <class GR>
 __device__ bool dilu_apply(const SolveArgs& a, const Mat<double>& A, const Mat<double>& AT, const double* rA,
-                           const double* rT, double* wA, double* wT, const Group& g, PhaseClock& pc)
+                           const double* rT, double* wA, double* wT, const GR& g, PhaseClock& pc)
 {
-    constexpr int G = 3;
+    constexpr int G = GR::wide ? 6 : 3;
     const RowIter it = rows_of(g);
     const int nlev = a.nlev, tail = min(a.tail_from, nlev);
     const int tid = (int)threadIdx.x, bs = (int)blockDim.x;
@@ -1361,13 +1585,57 @@ __device__ bool dilu_apply(const SolveArgs& a, const Mat<double>& A, const Mat<d
     return true;
 }
 
+// yA = A pA and yT = A^T pT over the thread's rows, sink(p, yA_p, yT_p).  On
+// the fixed-width layout both read a row's columns once; each sum in entry
+// order, as amul_row takes it.
+template <class GR, class Sink>
+__device__ __forceinline__ void dual_amul(const SolveArgs& a, const Mat<double>& A, const Mat<double>& AT,
+                                          const double* pA, const double* pT, const GR& g, Sink sink)
+{
+    const RowIter it = rows_of(g);
+    if (GR::wide && A.ell_w > 0 && A.ell_w <= 6) {
+        for (int p = it.first; p < a.n; p += it.stride) {
+            int c[6];
+            double u[6], w[6], xa[6], xt[6];
+#pragma unroll
+            for (int j = 0; j < 6; j++) {
+                const bool ok = j < A.ell_w;
+                const size_t e = (size_t)j * A.ell_stride + p;
+                c[j] = ok ? __ldcs(A.Ecol + e) : -1;
+                u[j] = ok ? __ldcs(A.Ea + e) : 0.0;
+                w[j] = ok ? __ldcs(AT.Ea + e) : 0.0;
+            }
+            const double d = __ldcs(A.d + p);
+            double ya = mul_rn(d, pA[p]), yt = mul_rn(d, pT[p]);
+#pragma unroll
+            for (int j = 0; j < 6; j++) {
+                xa[j] = c[j] >= 0 ? pA[c[j]] : 0.0;
+                xt[j] = c[j] >= 0 ? pT[c[j]] : 0.0;
+            }
+#pragma unroll
+            for (int j = 0; j < 6; j++)
+                if (c[j] >= 0) {
+                    ya = fmadd(u[j], xa[j], ya);
+                    yt = fmadd(w[j], xt[j], yt);
+                }
+            sink(p, ya, yt);
+        }
+        return;
+    }
+    for (int p = it.first; p < a.n; p += it.stride) {
+        const double ya = amul_row<double>(A, pA, p);
+        sink(p, ya, amul_row<double>(AT, pT, p));
+    }
+}
+
 // OpenFOAM PBiCG on an asymmetric matrix (the paper's momentum solver: PBiCG
 // with DILU), FP64, after phase_init (x, rA = b - A x, normFactor from the
 // row sums of A).  Vectors: x, rA = r, wA = w, pA = p, wT = q, rT = b (the
 // right-hand side is not needed past rT = b - A^T x), pT.  A^T shares A's
 // structure: its lower entries of row u hold upper_f and its upper entries of
 // row l lower_f; the transposed DILU sweeps use rD times those.
-__device__ bool solve_pbicg(const SolveArgs& a, const Group& g, double nfac, double res0, spuma_solver_perf& pf)
+template <class GR>
+__device__ bool solve_pbicg(const SolveArgs& a, const GR& g, double nfac, double res0, spuma_solver_perf& pf)
 {
     RowIter it = rows_of(g);
     const Mat<double> A = mat_of<double>(a);
@@ -1445,12 +1713,11 @@ __device__ bool solve_pbicg(const SolveArgs& a, const Group& g, double nfac, dou
             if (!group_sync(g)) return false;
             pc.lap(CK_PUPD);
             double acc[1] = {0.0};
-            for (int p = it.first; p < a.n; p += it.stride) {
-                const double y = amul_row<double>(A, pA, p);
-                wA[p] = y;
-                wT[p] = amul_row<double>(AT, pT, p);
-                acc[0] = fmadd(y, pT[p], acc[0]);
-            }
+            dual_amul(a, A, AT, pA, pT, g, [&](int p, double ya, double yt) {
+                wA[p] = ya;
+                wT[p] = yt;
+                acc[0] = fmadd(ya, pT[p], acc[0]);
+            });
             block_reduce_store<1>(acc, a.partials, SL_C, g.bid);
             if (!group_sync(g)) return false;
             grid_reduce_read<1>(acc, a.partials, SL_C, g.nblocks);
@@ -1479,8 +1746,8 @@ enum SolveKind { KIND_SETUP = 0, KIND_F64 = 1, KIND_MIXED = 2, KIND_MIXED_RESTAR
 // (batched launches); the single-system solver leaves it to the two small
 // kernels that follow it on the stream (k_true_residual_*), so that its own
 // register allocation is not burdened by one more Amul.
-template <int KIND, bool TRUE_INLINE>
-__device__ void run_system(const SolveArgs& a, const Group& g)
+template <int KIND, bool TRUE_INLINE, class GR>
+__device__ void run_system(const SolveArgs& a, const GR& g)
 {
     spuma_solver_perf pf;
     pf.initial_residual = 0.0;
@@ -1493,6 +1760,7 @@ __device__ void run_system(const SolveArgs& a, const Group& g)
     pf.status = 0;
     pf.n_levels = a.nlev;
     bool ok = true;
+    if constexpr (GR::wide) fill_chunk_table(a, g);
     if (a.mode == MODE_PREPARE || a.mode == MODE_SOLVE) {
         ok = phase_gather<KIND == KIND_PBICG>(a, g);
         if (ok) ok = phase_factor<KIND == KIND_PBICG>(a, g);
@@ -1562,10 +1830,26 @@ __device__ void run_system(const SolveArgs& a, const Group& g)
     }
 }
 
-template <int KIND>
-__global__ void __launch_bounds__(1024, 1) k_solve(SolveArgs a, unsigned long long timeout_ns)
+template <int MAXT>
+struct GroupOf {
+    using type = Group;
+};
+template <>
+struct GroupOf<512> {
+    using type = WideGroup;
+};
+
+// One instance per solve kind and largest block size (512 threads: 128
+// registers per thread; 1024: 64).
+template <int KIND, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) k_solve(SolveArgs a, unsigned long long timeout_ns)
 {
-    Group g{reinterpret_cast<unsigned long long*>(a.status + DS_BARRIER), a.status, (int)gridDim.x, (int)blockIdx.x, timeout_ns};
+    typename GroupOf<MAXT>::type g;
+    g.word = reinterpret_cast<unsigned long long*>(a.status + DS_BARRIER);
+    g.status = a.status;
+    g.nblocks = (int)gridDim.x;
+    g.bid = (int)blockIdx.x;
+    g.timeout_ns = timeout_ns;
     run_system<KIND, false>(a, g);
 }
 
@@ -1763,15 +2047,21 @@ static int kind_of(const SolveArgs& a)
     return KIND_F64;
 }
 
-static const void* solve_kernel(int kind)
+template <int MAXT>
+static const void* solve_kernel_t(int kind)
 {
     switch (kind) {
-    case KIND_SETUP: return (const void*)k_solve<KIND_SETUP>;
-    case KIND_MIXED: return (const void*)k_solve<KIND_MIXED>;
-    case KIND_MIXED_RESTART: return (const void*)k_solve<KIND_MIXED_RESTART>;
-    case KIND_PBICG: return (const void*)k_solve<KIND_PBICG>;
-    default: return (const void*)k_solve<KIND_F64>;
+    case KIND_SETUP: return (const void*)k_solve<KIND_SETUP, MAXT>;
+    case KIND_MIXED: return (const void*)k_solve<KIND_MIXED, MAXT>;
+    case KIND_MIXED_RESTART: return (const void*)k_solve<KIND_MIXED_RESTART, MAXT>;
+    case KIND_PBICG: return (const void*)k_solve<KIND_PBICG, MAXT>;
+    default: return (const void*)k_solve<KIND_F64, MAXT>;
     }
+}
+
+static const void* solve_kernel(int kind, int threads)
+{
+    return threads <= 512 ? solve_kernel_t<512>(kind) : solve_kernel_t<1024>(kind);
 }
 
 template <int MAXT>
@@ -1800,7 +2090,7 @@ int solve_blocks_per_sm(int threads, bool batch, int kind, size_t dyn = 0)
     const long long key = (((long long)(threads * 2 + (batch ? 1 : 0)) * 8 + kind) << 20) + (long long)dyn;
     auto it = g_occ.find(key);
     if (it != g_occ.end()) return it->second;
-    const void* k = batch ? batch_kernel(kind, threads) : solve_kernel(kind);
+    const void* k = batch ? batch_kernel(kind, threads) : solve_kernel(kind, threads);
     int nb = 0;
     cudaError_t e = cudaSuccess;
     if (dyn) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
@@ -1813,10 +2103,21 @@ int solve_blocks_per_sm(int threads, bool batch, int kind, size_t dyn = 0)
     return nb;
 }
 
-int default_threads(const spuma_solver_controls* ctl)
+// Threads per block of a single-system solve (block_threads 0).  Up to 512 the
+// kernels have 128 registers per thread and keep a round of sweep loads in
+// flight across the grid barriers (wide_sweep); 1024 threads keep more plain
+// rows in flight, which the largest meshes need.  Measured per iteration, DIC
+// FP64 / mixed, 256 | 512 | 1024 threads: 24^3 74 / 69 | 77 / 71 | 93 / 80 us,
+// 32^3 81 / 76 | 85 / 80 | 106 / 93, 64^3 123 / 111 | 116 / 104 | 153 / 130,
+// 100^3 181 / 140 | 176 / 135 | 196 / 161, 128^3 261 / 189 | 256 / 184 | 275 /
+// 193, 200^3 719 / 447 | 703 / 442 | 703 / 403; diagonal FP64 at 64^3 24 against
+// 30, at 128^3 91 against 93; PBiCG with DILU at 64^3 157 against 183, at 128^3
+// 394 against 380.
+int default_threads(const spuma_solver_controls* ctl, int64_t n, bool bicg = false)
 {
     if (ctl && ctl->block_threads > 0) return ctl->block_threads;
-    return 1024;
+    if (n <= 50000) return 256;
+    return n <= (bicg ? 1000000 : 3000000) ? 512 : 1024;
 }
 
 // Blocks of the persistent single-system solver: one per row chunk of
@@ -1874,7 +2175,7 @@ spuma_status launch_solve(spuma_ldu_t h, const SolveArgs& a, int threads, cudaSt
         SPUMA_CUDA(cudaMemsetAsync(b.phase_clk, 0, 8 * 256, s));
     }
     void* args[] = {(void*)&b, (void*)&tns};
-    SPUMA_CUDA(cudaLaunchCooperativeKernel(solve_kernel(kind), grid, threads, args, 0, s));
+    SPUMA_CUDA(cudaLaunchCooperativeKernel(solve_kernel(kind, threads), grid, threads, args, 0, s));
     count_launch();
     if (b.mode == MODE_SOLVE) {
         // the report's true residual (the solver's x in internal order is still in the workspace)
@@ -1961,7 +2262,7 @@ spuma_status pcg_solve_internal(spuma_ldu_t h, const double* diag, const double*
     a.b_orig = b;
     a.x_orig = x;
     a.perf = perf;
-    spuma_status st = launch_solve(h, a, default_threads(ctl), s);
+    spuma_status st = launch_solve(h, a, default_threads(ctl, h->n), s);
     if (st == SPUMA_OK) h->prepared_precond = ctl->precond;
     return st;
 }
@@ -2007,7 +2308,7 @@ spuma_status spuma_pbicg_solve(spuma_ldu_t h, const double* diag, const double* 
     a.x_orig = x;
     a.perf = perf;
     h->prepared_precond = -1;
-    return launch_solve(h, a, default_threads(ctl), s);
+    return launch_solve(h, a, default_threads(ctl, h->n, true), s);
 }
 
 spuma_status spuma_matrix_prepare(spuma_ldu_t h, const double* diag, const double* upper, int32_t precond,
