@@ -75,7 +75,8 @@ typedef enum {
  *    inner_rel_tol since the last update (or claims convergence, or max_iter
  *    is reached) the FP32 correction is added to the FP64 solution and the
  *    FP64 residual b - A x replaces the FP32 one; the search direction is
- *    kept (no Krylov restart).  max_iter bounds the FP32 iterations.
+ *    kept (no Krylov restart).  With DIC the FP32 PCG runs in Eisenstat's form
+ *    and follows its residual through the M^-1 norm.  max_iter bounds the FP32 iterations.
  *  precision SPUMA_MIXED_RESTART: FP64 iterative refinement around restarted
  *    FP32 inner solves: inner_rel_tol is the inner solve's relative
  *    tolerance, max_outer the maximum number of refinement steps, max_iter

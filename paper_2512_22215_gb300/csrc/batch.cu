@@ -20,7 +20,7 @@ SolveArgs make_args(spuma_ldu_t h);
 void fill_controls(SolveArgs& a, const spuma_solver_controls* ctl);
 bool ctl_ok(const spuma_solver_controls* c);
 int solve_blocks_per_sm(int threads, bool batch, int kind, size_t dyn = 0);
-int batch_kind(int precision);
+int batch_kind(int precision, int precond);
 spuma_status launch_batch_kernel(const BatchTable& t, int grid, int threads, int kind, cudaStream_t s);
 
 // Split `grid` blocks between systems in proportion to their weights, at
@@ -232,7 +232,7 @@ static spuma_status batch_create(int32_t n_sys, const spuma_ldu_t* hs, const dou
     cudaStream_t s = (cudaStream_t)stream;
     spuma_batch* bt = new spuma_batch();
     bt->n_sys = n_sys;
-    bt->kind = batch_kind(ctl->precision);
+    bt->kind = batch_kind(ctl->precision, ctl->precond);
     bt->hs.assign(hs, hs + n_sys);
     bt->args.resize(n_sys);
     auto fail = [&](spuma_status st) {

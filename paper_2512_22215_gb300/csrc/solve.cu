@@ -433,6 +433,10 @@ __device__ __forceinline__ void vadd_abs(A& acc, double2 r)
     acc.add(fabs(r.x));
     acc.add(fabs(r.y));
 }
+__device__ __forceinline__ float4 vsub(float4 x, float4 y)
+{
+    return make_float4(__fsub_rn(x.x, y.x), __fsub_rn(x.y, y.y), __fsub_rn(x.z, y.z), __fsub_rn(x.w, y.w));
+}
 __device__ __forceinline__ float4 vmul(float4 x, float4 y)
 {
     return make_float4(__fmul_rn(x.x, y.x), __fmul_rn(x.y, y.y), __fmul_rn(x.z, y.z), __fmul_rn(x.w, y.w));
@@ -614,80 +618,6 @@ __device__ bool phase_factor(const SolveArgs& a, const Group& g)
 }
 
 // ------------------------------------------------------ DIC sweeps ---------
-// Forward rows of one level: w = rD r - sum (rD a) w_lower (ascending face
-// order); with `rho` (top level: no upper neighbours, so w is final here)
-// also rho += w r.
-template <class T>
-__device__ __forceinline__ void fwd_rows(const Mat<T>& A, Vecs<T> v, int r0, int r1, int first, int stride, bool rho,
-                                         Acc<T>& arho)
-{
-    constexpr int R = ChainShape<T>::R, G = ChainShape<T>::G;
-    for (int pb = r0 + first; pb < r1; pb += R * stride) {
-        int p[R], e0[R], e1[R];
-        bool ok[R];
-        T ww[R], rr[R];
-#pragma unroll
-        for (int k = 0; k < R; k++) {
-            p[k] = pb + k * stride;
-            ok[k] = p[k] < r1;
-            e0[k] = ok[k] ? __ldcs(A.Lptr + p[k]) : 0;
-            e1[k] = ok[k] ? __ldcs(A.Lptr + p[k] + 1) : 0;
-            rr[k] = ok[k] ? v.r[p[k]] : T(0);
-            ww[k] = ok[k] ? mul_rn(__ldcs(A.rD + p[k]), rr[k]) : T(0);
-        }
-        rows_chain<T, R, G, false, true>(ww, e0, e1, A.Lcol, A.Lc, v.w);
-#pragma unroll
-        for (int k = 0; k < R; k++)
-            if (ok[k]) {
-                v.w[p[k]] = ww[k];
-                if (rho) arho.prod(ww[k], rr[k]);
-            }
-    }
-}
-
-// Backward rows of one level: w -= sum (rD a) w_upper (descending face
-// order); rho += w r.
-template <class T>
-__device__ __forceinline__ void bwd_rows(const Mat<T>& A, Vecs<T> v, int r0, int r1, int first, int stride,
-                                         Acc<T>& arho)
-{
-    constexpr int R = ChainShape<T>::R, G = ChainShape<T>::G;
-    // row extents one round ahead: the next round's are loaded while this
-    // round's entries and gathers are in flight (measured: backward sweep
-    // 135 -> 128 us per FP32 iteration at 200^3; no gain in the forward one)
-    int e0n[R], e1n[R];
-#pragma unroll
-    for (int k = 0; k < R; k++) {
-        const int pn = r0 + first + k * stride;
-        e0n[k] = pn < r1 ? __ldcs(A.Uptr + pn) : 0;
-        e1n[k] = pn < r1 ? __ldcs(A.Uptr + pn + 1) : 0;
-    }
-    for (int pb = r0 + first; pb < r1; pb += R * stride) {
-        int p[R], e0[R], e1[R];
-        bool ok[R];
-        T ww[R];
-#pragma unroll
-        for (int k = 0; k < R; k++) {
-            p[k] = pb + k * stride;
-            ok[k] = p[k] < r1;
-            e0[k] = ok[k] ? e0n[k] : 0;
-            e1[k] = ok[k] ? e1n[k] : 0;
-            const int pn = pb + (R + k) * stride;
-            e0n[k] = pn < r1 ? __ldcs(A.Uptr + pn) : 0;
-            e1n[k] = pn < r1 ? __ldcs(A.Uptr + pn + 1) : 0;
-        }
-#pragma unroll
-        for (int k = 0; k < R; k++) ww[k] = ok[k] ? v.w[p[k]] : T(0);
-        rows_chain<T, R, G, true, true>(ww, e0, e1, A.Ucol, A.Uc, v.w);
-#pragma unroll
-        for (int k = 0; k < R; k++)
-            if (ok[k]) {
-                v.w[p[k]] = ww[k];
-                arho.prod(ww[k], v.r[p[k]]);
-            }
-    }
-}
-
 // The block's contiguous chunk [c0, c1) of level L (sweep mapping 1):
 // the same 1/nblocks share of every level's Morton order, so a block's chunks
 // of consecutive levels cover nearly the same region of the mesh.
@@ -738,22 +668,70 @@ struct RoundIter {
     int L, pb, c1;
 };
 
-template <class T, int R, int G>
+template <class T, int R, int G, int NS>
 struct SweepRound {
     int e0[R], e1[R], c[R][G];
-    T cf[R][G], rr[R], ww[R];
+    T cf[R][G], s[R][NS];
 };
 
-// FWD: levels from .. to-1 ascending, else to-1 .. from descending.  SOLO: the
-// calling block takes whole levels by itself, with block barriers between them.
-template <class T, bool FWD, bool SOLO, class GR>
-__device__ __forceinline__ bool wide_sweep(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, const GR& g, PhaseClock& pc,
-                                           int from, int to, Acc<T>& arho, bool rho_last)
+// What a sweep loads of its own rows, starts the row's chain from and does with
+// the result, and the vector it gathers (which is also where results go).
+// w = rD r - sum c w_l; rho += w r at the top level (no upper neighbours there:
+// w is final).
+template <class T>
+struct FwdR {
+    static constexpr int NS = 2;
+    const T *r, *rD;
+    T* w;
+    Acc<T>& rho;
+    int top;
+    __device__ __forceinline__ const T* vec() const { return w; }
+    __device__ __forceinline__ void load(int p, T (&s)[NS]) const
+    {
+        s[0] = r[p];
+        s[1] = __ldcs(rD + p);
+    }
+    __device__ __forceinline__ T init(T (&s)[NS]) const { return mul_rn(s[1], s[0]); }
+    __device__ __forceinline__ void store(int p, T v, const T (&s)[NS], int L) const
+    {
+        w[p] = v;
+        if (L == top) rho.prod(v, s[0]);
+    }
+};
+// w -= sum c w_u; rho += w r.
+template <class T>
+struct BwdR {
+    static constexpr int NS = 2;
+    const T* r;
+    T* w;
+    Acc<T>& rho;
+    __device__ __forceinline__ const T* vec() const { return w; }
+    __device__ __forceinline__ void load(int p, T (&s)[NS]) const
+    {
+        s[0] = r[p];
+        s[1] = w[p];
+    }
+    __device__ __forceinline__ T init(T (&s)[NS]) const { return s[1]; }
+    __device__ __forceinline__ void store(int p, T v, const T (&s)[NS], int) const
+    {
+        w[p] = v;
+        rho.prod(v, s[0]);
+    }
+};
+
+// Levels from .. to-1 ascending (FWD) or to-1 .. from descending, one grid
+// barrier after each (after the last one too unless !last_sync).  SOLO: the
+// calling block takes whole levels by itself, with block barriers.  `at_last`
+// runs before the last level's barrier (a reduction's partials).
+template <class T, bool FWD, bool SOLO, class GR, class Op, class Last>
+__device__ __forceinline__ bool wide_sweep(const SolveArgs& a, const Mat<T>& A, const GR& g, PhaseClock& pc, int from,
+                                           int to, bool last_sync, const Op& op, Last at_last)
 {
-    constexpr int R = WideShape<T>::R, G = WideShape<T>::G;
-    // blocks of one warp keep it at work
-    const int service = !SOLO && blockDim.x > kWarp ? kWarp : 0;
-    const int nlev = a.nlev, tid = (int)threadIdx.x - service, bs = (int)blockDim.x - service;
+    constexpr int R = WideShape<T>::R, G = WideShape<T>::G, NS = Op::NS;
+    using Round = SweepRound<T, R, G, NS>;
+    // blocks of up to three warps keep it at work
+    const int service = !SOLO && blockDim.x >= 4 * kWarp ? kWarp : 0;
+    const int tid = (int)threadIdx.x - service, bs = (int)blockDim.x - service;
     const bool chunks = !SOLO && a.sweep != 0, own = SOLO || chunks;
     const int first = own ? tid : g.bid * bs + tid, stride = own ? bs : g.nblocks * bs;
     const int2* table = chunk_table();
@@ -795,18 +773,13 @@ __device__ __forceinline__ bool wide_sweep(const SolveArgs& a, const Mat<T>& A, 
             e1[k] = ok ? __ldcs(ptr + p + 1) : 0;
         }
     };
-    auto entries = [&](const RoundIter& it, SweepRound<T, R, G>& q) {
+    auto entries = [&](const RoundIter& it, Round& q) {
 #pragma unroll
         for (int k = 0; k < R; k++) {
             const int p = it.pb + k * stride;
-            const bool ok = it.L != Lend && p < it.c1;
-            if (FWD) {
-                q.rr[k] = ok ? v.r[p] : T(0);
-                q.ww[k] = ok ? __ldcs(A.rD + p) : T(0);
-            } else {
-                q.ww[k] = ok ? v.w[p] : T(0);
-                q.rr[k] = ok ? v.r[p] : T(0);
-            }
+#pragma unroll
+            for (int j = 0; j < NS; j++) q.s[k][j] = T(0);
+            if (it.L != Lend && p < it.c1) op.load(p, q.s[k]);
 #pragma unroll
             for (int j = 0; j < G; j++) {
                 const int e = FWD ? q.e0[k] + j : q.e1[k] - 1 - j;
@@ -817,7 +790,7 @@ __device__ __forceinline__ bool wide_sweep(const SolveArgs& a, const Mat<T>& A, 
         }
     };
     RoundIter cur{Lbeg, 0, 0}, nxt, nn;
-    SweepRound<T, R, G> q, qn;
+    Round q, qn;
     int n0[R], n1[R];
     open(cur);
     nxt = cur;
@@ -829,11 +802,11 @@ __device__ __forceinline__ bool wide_sweep(const SolveArgs& a, const Mat<T>& A, 
         while (cur.L == L) {
             // this round's gathers, then the entries of the next round and the
             // extents of the one after
-            T x[R][G], acc[R];
+            T x[R][G];
 #pragma unroll
             for (int k = 0; k < R; k++)
 #pragma unroll
-                for (int j = 0; j < G; j++) x[k][j] = q.c[k][j] >= 0 ? gather<true>(v.w, q.c[k][j], pol) : T(0);
+                for (int j = 0; j < G; j++) x[k][j] = q.c[k][j] >= 0 ? gather<true>(op.vec(), q.c[k][j], pol) : T(0);
 #pragma unroll
             for (int k = 0; k < R; k++) {
                 qn.e0[k] = n0[k];
@@ -845,19 +818,16 @@ __device__ __forceinline__ bool wide_sweep(const SolveArgs& a, const Mat<T>& A, 
             extents(nn, n0, n1);
 #pragma unroll
             for (int k = 0; k < R; k++) {
-                acc[k] = FWD ? mul_rn(q.ww[k], q.rr[k]) : q.ww[k];
+                T acc = op.init(q.s[k]);
 #pragma unroll
                 for (int j = 0; j < G; j++)
-                    if (q.c[k][j] >= 0) acc[k] = fmadd(-q.cf[k][j], x[k][j], acc[k]);
+                    if (q.c[k][j] >= 0) acc = fmadd(-q.cf[k][j], x[k][j], acc);
                 for (int j = G; j < q.e1[k] - q.e0[k]; j++) {   // rows of more than G entries
                     const int e = FWD ? q.e0[k] + j : q.e1[k] - 1 - j;
-                    acc[k] = fmadd(-__ldcs(coef + e), v.w[__ldcs(col + e)], acc[k]);
+                    acc = fmadd(-__ldcs(coef + e), op.vec()[__ldcs(col + e)], acc);
                 }
                 const int p = cur.pb + k * stride;
-                if (p < cur.c1) {
-                    v.w[p] = acc[k];
-                    if (!FWD || L == nlev - 1) arho.prod(acc[k], q.rr[k]);   // top level: w is final here
-                }
+                if (p < cur.c1) op.store(p, acc, q.s[k], L);
             }
             cur = nxt;
             q = qn;
@@ -867,9 +837,9 @@ __device__ __forceinline__ bool wide_sweep(const SolveArgs& a, const Mat<T>& A, 
             __syncthreads();
             continue;
         }
-        if (rho_last && (FWD ? L == nlev - 1 : L == 0)) {
-            double t[1] = {arho.value()};
-            block_reduce_store<1>(t, a.partials, SL_B, g.bid);
+        if (L + (FWD ? 1 : -1) == Lend) {
+            at_last();
+            if (!last_sync) return true;
         }
         if (!group_sync(g)) return false;
         pc.lap((FWD ? CK_FWD : CK_BWD) + min(L, 63));
@@ -877,88 +847,129 @@ __device__ __forceinline__ bool wide_sweep(const SolveArgs& a, const Mat<T>& A, 
     return true;
 }
 
-// w = M^-1 r with the DIC (or DILU) factor held in A's sweep coefficients,
-// and the block partials of rho = w.r in SL_B before the last grid
-// barrier.  Forward sweep over levels 0 .. nlev-1, backward over nlev-2 .. 0
-// (the top level has no upper neighbours: its backward step would leave w
-// as it is, so its rho terms are taken in the forward step), one grid
-// barrier per level.  The small last levels (level >= tail_from) run on the
-// group's first block alone, forward then backward, with block-level
-// barriers and one grid barrier after them.
-// Row mapping (a.sweep): 1 (default), each block sweeps one contiguous chunk
-// of every level (the same 1/nblocks share of each level's Morton order);
-// 0, a level's rows strided over the group in blockDim-row pieces.  Measured
-// at 200^3: mixed solve 328.8 against 333.5 ms, FP64 582.5 against 599.7 ms.
+// One level's rows [r0, r1) from `first` with `stride` without the loads ahead
+// (Group: 64 registers): extents one round ahead, entries in groups of G, R
+// rows in lockstep.
+template <class T, bool FWD, class Op>
+__device__ __forceinline__ void level_rows(const Mat<T>& A, const Op& op, int r0, int r1, int first, int stride, int L)
+{
+    constexpr int R = ChainShape<T>::R, G = ChainShape<T>::G;
+    const int* ptr = FWD ? A.Lptr : A.Uptr;
+    int e0n[R], e1n[R];
+#pragma unroll
+    for (int k = 0; k < R; k++) {
+        const int pn = r0 + first + k * stride;
+        e0n[k] = pn < r1 ? __ldcs(ptr + pn) : 0;
+        e1n[k] = pn < r1 ? __ldcs(ptr + pn + 1) : 0;
+    }
+    for (int pb = r0 + first; pb < r1; pb += R * stride) {
+        int e0[R], e1[R];
+        T v[R], s[R][Op::NS];
+#pragma unroll
+        for (int k = 0; k < R; k++) {
+            const int p = pb + k * stride, pn = p + R * stride;
+            e0[k] = e0n[k];
+            e1[k] = e1n[k];
+            e0n[k] = pn < r1 ? __ldcs(ptr + pn) : 0;
+            e1n[k] = pn < r1 ? __ldcs(ptr + pn + 1) : 0;
+#pragma unroll
+            for (int j = 0; j < Op::NS; j++) s[k][j] = T(0);
+            if (p < r1) op.load(p, s[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < R; k++) v[k] = op.init(s[k]);
+        rows_chain<T, R, G, !FWD, true>(v, e0, e1, FWD ? A.Lcol : A.Ucol, FWD ? A.Lc : A.Uc, op.vec());
+#pragma unroll
+        for (int k = 0; k < R; k++)
+            if (pb + k * stride < r1) op.store(pb + k * stride, v[k], s[k], L);
+    }
+}
+
+// Levels from .. to-1 (FWD ascending, else descending) over the grid, one
+// barrier after each (the last one's only with last_sync).  Row mapping
+// (a.sweep): 1 (default), each block sweeps one contiguous chunk of every level
+// (the same 1/nblocks share of each level's Morton order); 0, a level's rows
+// strided over the group in blockDim-row pieces.  Measured at 200^3: mixed
+// solve 328.8 against 333.5 ms, FP64 582.5 against 599.7 ms.
+template <class T, bool FWD, class GR, class Op, class Last>
+__device__ __forceinline__ bool sweep_levels(const SolveArgs& a, const Mat<T>& A, const GR& g, PhaseClock& pc, int from,
+                                             int to, bool last_sync, const Op& op, Last at_last)
+{
+    if constexpr (GR::wide) {
+        return wide_sweep<T, FWD, false>(a, A, g, pc, from, to, last_sync, op, at_last);
+    } else {
+        const RowIter it = rows_of(g);
+        const int Lend = FWD ? to : from - 1;
+        for (int L = FWD ? from : to - 1; L != Lend; L += FWD ? 1 : -1) {
+            int c0, c1;
+            if (a.sweep != 0) {
+                level_chunk(a.lvl, L, g.nblocks, g.bid, c0, c1);
+                level_rows<T, FWD>(A, op, c0, c1, (int)threadIdx.x, (int)blockDim.x, L);
+            } else {
+                level_rows<T, FWD>(A, op, a.lvl[L], a.lvl[L + 1], it.first, it.stride, L);
+            }
+            if (L + (FWD ? 1 : -1) == Lend) {
+                at_last();
+                if (!last_sync) return true;
+            }
+            if (!group_sync(g)) return false;
+            pc.lap((FWD ? CK_FWD : CK_BWD) + min(L, 63));
+        }
+        return true;
+    }
+}
+
+// The small last levels from .. to-1 on the group's first block alone.
+template <class T, bool FWD, class GR, class Op>
+__device__ __forceinline__ void sweep_solo(const SolveArgs& a, const Mat<T>& A, const GR& g, PhaseClock& pc, int from,
+                                           int to, const Op& op)
+{
+    if constexpr (GR::wide) {
+        wide_sweep<T, FWD, true>(a, A, g, pc, from, to, true, op, [] {});
+    } else {
+        for (int L = FWD ? from : to - 1; L != (FWD ? to : from - 1); L += FWD ? 1 : -1) {
+            level_rows<T, FWD>(A, op, a.lvl[L], a.lvl[L + 1], (int)threadIdx.x, (int)blockDim.x, L);
+            __syncthreads();
+        }
+    }
+}
+
+// w = M^-1 r with the DIC factor held in A's sweep coefficients, and the block
+// partials of rho = w.r in SL_B before the last grid barrier.  Forward sweep
+// over levels 0 .. nlev-1, backward over nlev-2 .. 0 (the top level has no
+// upper neighbours: its backward step would leave w as it is, so its rho terms
+// are taken in the forward step), one grid barrier per level.  The small last
+// levels (level >= tail_from) run on the group's first block alone, forward
+// then backward, with block-level barriers and one grid barrier after them.
 template <class T, class GR>
 __device__ bool dic_apply(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, const GR& g, PhaseClock& pc)
 {
-    const RowIter it = rows_of(g);
     const int nlev = a.nlev, tail = min(a.tail_from, nlev);
-    const int tid = (int)threadIdx.x, bs = (int)blockDim.x;
     Acc<T> arho;
-    auto end_step = [&](bool last) {
-        if (last) {
-            double t[1] = {arho.value()};
-            block_reduce_store<1>(t, a.partials, SL_B, g.bid);
-        }
+    auto rho_partials = [&] {
+        double t[1] = {arho.value()};
+        block_reduce_store<1>(t, a.partials, SL_B, g.bid);
+    };
+    if (nlev == 0) {
+        rho_partials();
         return group_sync(g);
-    };
-    if (nlev == 0) return end_step(true);
-    const bool chunks = a.sweep != 0;
-    auto rows = [&](int L, int& c0, int& c1, int& first, int& stride) {
-        if (chunks) {
-            level_chunk(a.lvl, L, g.nblocks, g.bid, c0, c1);
-            first = tid;
-            stride = bs;
-        } else {
-            c0 = a.lvl[L];
-            c1 = a.lvl[L + 1];
-            first = it.first;
-            stride = it.stride;
-        }
-    };
-    if constexpr (GR::wide) {
-        if (!wide_sweep<T, true, false>(a, A, v, g, pc, 0, tail, arho, nlev == 1)) return false;
-    } else {
-        for (int L = 0; L < tail; L++) {
-            int c0, c1, first, stride;
-            rows(L, c0, c1, first, stride);
-            fwd_rows<T>(A, v, c0, c1, first, stride, L == nlev - 1, arho);
-            if (!end_step(nlev == 1)) return false;
-            pc.lap(CK_FWD + min(L, 63));
-        }
     }
+    const FwdR<T> fwd{v.r, A.rD, v.w, arho, nlev - 1};
+    const BwdR<T> bwd{v.r, v.w, arho};
+    if (!sweep_levels<T, true>(a, A, g, pc, 0, tail, true, fwd, [&] {
+            if (nlev == 1) rho_partials();
+        }))
+        return false;
     if (tail < nlev) {
         if (g.bid == 0) {
-            if constexpr (GR::wide) {
-                wide_sweep<T, true, true>(a, A, v, g, pc, tail, nlev, arho, false);
-                wide_sweep<T, false, true>(a, A, v, g, pc, tail, nlev - 1, arho, false);
-            } else {
-                for (int L = tail; L < nlev; L++) {
-                    fwd_rows<T>(A, v, a.lvl[L], a.lvl[L + 1], tid, bs, L == nlev - 1, arho);
-                    __syncthreads();
-                }
-                for (int L = nlev - 2; L >= tail; L--) {
-                    bwd_rows<T>(A, v, a.lvl[L], a.lvl[L + 1], tid, bs, arho);
-                    __syncthreads();
-                }
-            }
+            sweep_solo<T, true>(a, A, g, pc, tail, nlev, fwd);
+            sweep_solo<T, false>(a, A, g, pc, tail, nlev - 1, bwd);
         }
-        if (!end_step(tail == 0)) return false;
+        if (tail == 0) rho_partials();
+        if (!group_sync(g)) return false;
         pc.lap(CK_FWD + min(tail, 63));
     }
-    if constexpr (GR::wide) {
-        return wide_sweep<T, false, false>(a, A, v, g, pc, 0, min(tail, nlev - 1), arho, true);
-    } else {
-        for (int L = min(tail, nlev - 1) - 1; L >= 0; L--) {
-            int c0, c1, first, stride;
-            rows(L, c0, c1, first, stride);
-            bwd_rows<T>(A, v, c0, c1, first, stride, arho);
-            if (!end_step(L == 0)) return false;
-            pc.lap(CK_BWD + min(L, 63));
-        }
-    }
-    return true;
+    return sweep_levels<T, false>(a, A, g, pc, 0, min(tail, nlev - 1), true, bwd, rho_partials);
 }
 
 // ----------------------------------------------------- streaming passes ---
@@ -1324,6 +1335,225 @@ __device__ bool solve_mixed_reliable(const SolveArgs& a, const GR& g, double nfa
     // the FP32 w and p were gathered evict-last: hand their lines back
     release_lines(a.wi, 4 * (size_t)a.n, it.first, it.stride);
     release_lines(a.pi, 4 * (size_t)a.n, it.first, it.stride);
+    pf.initial_residual = res0;
+    pf.final_residual = res;
+    pf.n_iter = n_it;
+    pf.n_outer = updates;
+    pf.converged = converged(res, res0, a.tol, a.rel_tol);
+    pf.singular = singular;
+    return ok;
+}
+
+// The same reliable updates for DIC, with Eisenstat's form of the inner PCG (S.
+// C. Eisenstat, "Efficient implementation of a class of preconditioned conjugate
+// gradient methods", SIAM J. Sci. Stat. Comput. 2, 1981).  M = (P + L) P^-1 (P +
+// U) shares A's off-diagonal, A = L + D + U, so the product A p follows from the
+// two sweeps and no Amul is needed.  With y = (P + L)^-1 r (kept in place of r),
+// the search direction's image t = P^-1 (P + U) p:
+//   rho = y.P y;  t = y + beta t;  p = t - P^-1 U p           (backward sweep)
+//   h = p - (P + L)^-1 A p = (2 - D/P) p - t - P^-1 L h        (forward sweep)
+//   sigma = p.A p = (P t).(p - h);  alpha = rho/sigma
+//   x += alpha p;  y -= alpha (p - h)
+// the same iterates in exact arithmetic.  An iteration reads 16F + 72N bytes
+// instead of 36F + 76N and has two grid barriers fewer: 200^3 402 -> 330 us,
+// 128^3 181 -> 146, 64^3 100 -> 92 per iteration; 1142 iterations to 1e-11 at
+// 200^3 against 1138 with the product.  sum|r|, which decides
+// when the FP64 residual is taken, is followed by kappa sqrt(rho): kappa = sum|r|
+// / sqrt(rho) at the last FP64 residual (it moves by 2-3 % between them once the
+// first digits are gone: 24^3 and 48^3, log-normal diffusivity); whether the
+// solve has converged is decided on the FP64 residual alone, as above.
+struct FwdY {   // y = rD r - sum c y_l; rho += y (P y)
+    static constexpr int NS = 3;
+    const float *r, *rD, *P;
+    float* y;
+    Acc<float>& rho;
+    __device__ __forceinline__ const float* vec() const { return y; }
+    __device__ __forceinline__ void load(int p, float (&s)[NS]) const
+    {
+        s[0] = r[p];
+        s[1] = __ldcs(rD + p);
+        s[2] = __ldcs(P + p);
+    }
+    __device__ __forceinline__ float init(float (&s)[NS]) const { return __fmul_rn(s[1], s[0]); }
+    __device__ __forceinline__ void store(int p, float v, const float (&s)[NS], int) const
+    {
+        y[p] = v;
+        rho.prod(__fmul_rn(s[2], v), v);
+    }
+};
+struct BwdP {   // t = y + beta t; p = t - sum c p_u
+    static constexpr int NS = 2;
+    const float* y;
+    float *t, *p;
+    float beta;
+    bool first;
+    __device__ __forceinline__ const float* vec() const { return p; }
+    __device__ __forceinline__ void load(int i, float (&s)[NS]) const
+    {
+        s[0] = y[i];
+        s[1] = first ? 0.0f : __ldcs(t + i);
+    }
+    __device__ __forceinline__ float init(float (&s)[NS]) const { return s[1] = first ? s[0] : __fmaf_rn(beta, s[1], s[0]); }
+    __device__ __forceinline__ void store(int i, float v, const float (&s)[NS], int) const
+    {
+        t[i] = s[1];
+        p[i] = v;
+    }
+};
+struct FwdH {   // h = e p - t - sum c h_l; sigma += (P t)(p - h)
+    static constexpr int NS = 4;
+    const float *p, *t, *e, *P;
+    float* h;
+    Acc<float>& sigma;
+    __device__ __forceinline__ const float* vec() const { return h; }
+    __device__ __forceinline__ void load(int i, float (&s)[NS]) const
+    {
+        s[0] = p[i];
+        s[1] = t[i];
+        s[2] = __ldcs(e + i);
+        s[3] = __ldcs(P + i);
+    }
+    __device__ __forceinline__ float init(float (&s)[NS]) const { return __fmaf_rn(s[2], s[0], -s[1]); }
+    __device__ __forceinline__ void store(int i, float v, const float (&s)[NS], int) const
+    {
+        h[i] = v;
+        sigma.prod(__fmul_rn(s[3], s[1]), __fsub_rn(s[0], v));
+    }
+};
+
+template <class GR>
+__device__ bool solve_mixed_eisenstat(const SolveArgs& a, const GR& g, double nfac, double res0, spuma_solver_perf& pf)
+{
+    RowIter it = rows_of(g);
+    const Mat<float> A = mat_of<float>(a);
+    PhaseClock pc(a.phase_clk, g.bid);
+    // t, e = 2 - D/P and P live in FP64 vectors that the mixed forms do not use
+    float *x = a.xi, *r = a.ri, *y = a.wi, *p = a.pi, *h = a.qi;
+    float *t = reinterpret_cast<float*>(a.p), *e = reinterpret_cast<float*>(a.w), *P = reinterpret_cast<float*>(a.q);
+    const int nlev = a.nlev, tail = min(a.tail_from, nlev), nv = a.n / 4;
+    const double delta = a.inner_rel_tol;
+    // partials of one sum, the barrier, the grid's value
+    auto total = [&](Acc<float>& acc, int slot, double* out) {
+        double v[1] = {acc.value()};
+        block_reduce_store<1>(v, a.partials, slot, g.bid);
+        if (!group_sync(g)) return false;
+        grid_reduce_read<1>(v, a.partials, slot, g.nblocks);
+        *out = v[0];
+        return true;
+    };
+    auto read = [&](int slot, double* out) {
+        double v[1];
+        grid_reduce_read<1>(v, a.partials, slot, g.nblocks);
+        *out = v[0];
+    };
+    auto partials = [&](Acc<float>& acc, int slot) {
+        double v[1] = {acc.value()};
+        block_reduce_store<1>(v, a.partials, slot, g.bid);
+    };
+    auto forward_r = [&](double* rho) {
+        Acc<float> acc;
+        const FwdY op{r, A.rD, P, y, acc};
+        if (!sweep_levels<float, true>(a, A, g, pc, 0, tail, true, op, [&] {
+                if (tail == nlev) partials(acc, SL_B);
+            }))
+            return false;
+        if (tail < nlev) {
+            if (g.bid == 0) sweep_solo<float, true>(a, A, g, pc, tail, nlev, op);
+            return total(acc, SL_B, rho);
+        }
+        read(SL_B, rho);
+        return true;
+    };
+    auto directions = [&](bool first, float beta, double* sigma) {
+        const BwdP bwd{y, t, p, beta, first};
+        if (tail < nlev) {
+            if (g.bid == 0) sweep_solo<float, false>(a, A, g, pc, tail, nlev, bwd);
+            if (!group_sync(g)) return false;
+            pc.lap(CK_BWD + min(tail, 63));
+        }
+        // no barrier between the backward and the forward step of level 0: a
+        // row's p and t are its own thread's
+        if (!sweep_levels<float, false>(a, A, g, pc, 0, tail, false, bwd, [] {})) return false;
+        Acc<float> acc;
+        const FwdH fwd{p, t, e, P, h, acc};
+        if (!sweep_levels<float, true>(a, A, g, pc, 0, tail, true, fwd, [&] {
+                if (tail == nlev) partials(acc, SL_C);
+            }))
+            return false;
+        if (tail < nlev) {
+            if (g.bid == 0) sweep_solo<float, true>(a, A, g, pc, tail, nlev, fwd);
+            const bool ok = total(acc, SL_C, sigma);
+            pc.lap(CK_FWD + min(tail, 63));
+            return ok;
+        }
+        read(SL_C, sigma);
+        return true;
+    };
+    double res = res0, rupd = res0;
+    int n_it = 0, updates = 0, singular = 0;
+    bool ok = true;
+    if (!converged(res0, res0, a.tol, a.rel_tol)) {
+        for (int i = it.first; i < a.n; i += it.stride) {
+            const double rd = a.rD64[i];
+            P[i] = (float)__ddiv_rn(1.0, rd);
+            e[i] = (float)__fma_rn(-rd, a.d64[i], 2.0);
+            r[i] = (float)a.r[i];
+            x[i] = 0.0f;
+        }
+        if (!group_sync(g)) return false;
+        double rho, rho_old = 1.0;
+        if (!forward_r(&rho)) return false;
+        double kappa = res / sqrt(rho);
+        for (bool first = true;; first = false) {
+            double sigma;
+            if (!directions(first, first ? 0.0f : (float)(rho / rho_old), &sigma)) return false;
+            pc.count(CK_ITERS);
+            double rs, rm;
+            if (fabs(sigma) / nfac < 1e-300) {
+                singular = 1;
+                ok = refine_residual(a, g, true, &rs, &rm);
+                res = rs / nfac;
+                break;
+            }
+            const float alpha = (float)(rho / sigma);
+            // x += alpha p, y -= alpha (p - h), rho = y.P y
+            Acc<float> acc;
+            float4 *x4 = reinterpret_cast<float4*>(x), *y4 = reinterpret_cast<float4*>(y);
+            const float4 *p4 = reinterpret_cast<const float4*>(p), *h4 = reinterpret_cast<const float4*>(h);
+            const float4* P4 = reinterpret_cast<const float4*>(P);
+            for (int i = it.first; i < nv; i += it.stride) {
+                const float4 pp = p4[i], gg = vsub(pp, __ldcs(h4 + i));
+                const float4 yy = vfma(-alpha, gg, y4[i]);
+                __stcs(x4 + i, vfma(alpha, pp, __ldcs(x4 + i)));
+                y4[i] = yy;
+                vprod(acc, vmul(__ldcs(P4 + i), yy), yy);
+            }
+            for (int i = 4 * nv + it.first; i < a.n; i += it.stride) {
+                const float yy = __fmaf_rn(-alpha, __fsub_rn(p[i], h[i]), y[i]);
+                x[i] = __fmaf_rn(alpha, p[i], x[i]);
+                y[i] = yy;
+                acc.prod(__fmul_rn(P[i], yy), yy);
+            }
+            rho_old = rho;
+            if (!total(acc, SL_D, &rho)) return false;
+            pc.lap(CK_UPD);
+            n_it++;
+            const double est = kappa * sqrt(rho);
+            if (!(est < delta * rupd || converged(est, res0, a.tol, a.rel_tol) || n_it >= a.max_iter)) continue;
+            if (!refine_residual(a, g, true, &rs, &rm)) return false;
+            pc.lap(CK_RESID);
+            updates++;
+            res = rs / nfac;
+            if (converged(res, res0, a.tol, a.rel_tol) || n_it >= a.max_iter) break;
+            rupd = res;
+            if (!forward_r(&rho)) return false;
+            kappa = res / sqrt(rho);
+        }
+    }
+    // y, p and h were gathered evict-last: hand their lines back
+    release_lines(y, 4 * (size_t)a.n, it.first, it.stride);
+    release_lines(p, 4 * (size_t)a.n, it.first, it.stride);
+    release_lines(h, 4 * (size_t)a.n, it.first, it.stride);
     pf.initial_residual = res0;
     pf.final_residual = res;
     pf.n_iter = n_it;
@@ -1740,7 +1970,7 @@ __device__ bool solve_pbicg(const SolveArgs& a, const GR& g, double nfac, double
     return true;
 }
 
-enum SolveKind { KIND_SETUP = 0, KIND_F64 = 1, KIND_MIXED = 2, KIND_MIXED_RESTART = 3, KIND_PBICG = 4 };
+enum SolveKind { KIND_SETUP = 0, KIND_F64 = 1, KIND_MIXED = 2, KIND_MIXED_RESTART = 3, KIND_PBICG = 4, KIND_MIXED_DIC = 5 };
 
 // TRUE_INLINE: the report's true residual is computed inside the launch
 // (batched launches); the single-system solver leaves it to the two small
@@ -1794,6 +2024,8 @@ __device__ void run_system(const SolveArgs& a, const GR& g)
                     ok = solve_pbicg(a, g, nfac, res0, pf);
                 } else if constexpr (KIND == KIND_MIXED) {
                     ok = solve_mixed_reliable(a, g, nfac, res0, pf);
+                } else if constexpr (KIND == KIND_MIXED_DIC) {
+                    ok = solve_mixed_eisenstat(a, g, nfac, res0, pf);
                 } else if constexpr (KIND == KIND_MIXED_RESTART) {
                     ok = solve_mixed_restart(a, g, nfac, pf);
                 } else {
@@ -1891,8 +2123,12 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 2 : 1) k_solve_batch(Batch
     while (s + 1 < t.n_sys && (int)blockIdx.x >= t.split[s + 1]) s++;
     if (threadIdx.x == 0) sa = *t.args[s];
     __syncthreads();
-    Group g{reinterpret_cast<unsigned long long*>(sa.status + DS_BARRIER), sa.status, t.split[s + 1] - t.split[s],
-            (int)blockIdx.x - t.split[s], timeout_ns};
+    typename GroupOf<(MAXT <= 512 ? 512 : 1024)>::type g;
+    g.word = reinterpret_cast<unsigned long long*>(sa.status + DS_BARRIER);
+    g.status = sa.status;
+    g.nblocks = t.split[s + 1] - t.split[s];
+    g.bid = (int)blockIdx.x - t.split[s];
+    g.timeout_ns = timeout_ns;
     run_system<KIND, true>(sa, g);
 }
 
@@ -2038,13 +2274,17 @@ SolveArgs make_args(spuma_ldu_t h)
     return a;
 }
 
+static int precision_kind(int precision, int precond)
+{
+    if (precision == SPUMA_MIXED) return precond == SPUMA_PRECOND_DIC ? KIND_MIXED_DIC : KIND_MIXED;
+    return precision == SPUMA_MIXED_RESTART ? KIND_MIXED_RESTART : KIND_F64;
+}
+
 static int kind_of(const SolveArgs& a)
 {
     if (a.mode != MODE_SOLVE) return KIND_SETUP;
     if (a.lower_orig) return KIND_PBICG;
-    if (a.precision == SPUMA_MIXED) return KIND_MIXED;
-    if (a.precision == SPUMA_MIXED_RESTART) return KIND_MIXED_RESTART;
-    return KIND_F64;
+    return precision_kind(a.precision, a.precond);
 }
 
 template <int MAXT>
@@ -2053,6 +2293,7 @@ static const void* solve_kernel_t(int kind)
     switch (kind) {
     case KIND_SETUP: return (const void*)k_solve<KIND_SETUP, MAXT>;
     case KIND_MIXED: return (const void*)k_solve<KIND_MIXED, MAXT>;
+    case KIND_MIXED_DIC: return (const void*)k_solve<KIND_MIXED_DIC, MAXT>;
     case KIND_MIXED_RESTART: return (const void*)k_solve<KIND_MIXED_RESTART, MAXT>;
     case KIND_PBICG: return (const void*)k_solve<KIND_PBICG, MAXT>;
     default: return (const void*)k_solve<KIND_F64, MAXT>;
@@ -2069,6 +2310,7 @@ static const void* batch_kernel_t(int kind)
 {
     switch (kind) {
     case KIND_MIXED: return (const void*)k_solve_batch<KIND_MIXED, MAXT>;
+    case KIND_MIXED_DIC: return (const void*)k_solve_batch<KIND_MIXED_DIC, MAXT>;
     case KIND_MIXED_RESTART: return (const void*)k_solve_batch<KIND_MIXED_RESTART, MAXT>;
     default: return (const void*)k_solve_batch<KIND_F64, MAXT>;
     }
@@ -2105,19 +2347,19 @@ int solve_blocks_per_sm(int threads, bool batch, int kind, size_t dyn = 0)
 
 // Threads per block of a single-system solve (block_threads 0).  Up to 512 the
 // kernels have 128 registers per thread and keep a round of sweep loads in
-// flight across the grid barriers (wide_sweep); 1024 threads keep more plain
-// rows in flight, which the largest meshes need.  Measured per iteration, DIC
-// FP64 / mixed, 256 | 512 | 1024 threads: 24^3 74 / 69 | 77 / 71 | 93 / 80 us,
-// 32^3 81 / 76 | 85 / 80 | 106 / 93, 64^3 123 / 111 | 116 / 104 | 153 / 130,
-// 100^3 181 / 140 | 176 / 135 | 196 / 161, 128^3 261 / 189 | 256 / 184 | 275 /
-// 193, 200^3 719 / 447 | 703 / 442 | 703 / 403; diagonal FP64 at 64^3 24 against
-// 30, at 128^3 91 against 93; PBiCG with DILU at 64^3 157 against 183, at 128^3
-// 394 against 380.
+// flight across the grid barriers (wide_sweep).  Measured per iteration, DIC
+// FP64 / mixed, 256 | 512 | 1024 threads: 24^3 73 / 63 | 76 / 64 | 92 / 82 us,
+// 32^3 80 / 69 | 84 / 73 | 104 / 93, 64^3 119 / 98 | 112 / 92 | 151 / 131,
+// 100^3 175 / 114 | 171 / 110 | 195 / 153, 128^3 257 / 149 | 251 / 146 | 274 /
+// 174, 200^3 709 / 333 | 692 / 330 | 702 / 336; diagonal FP64 at 64^3 24 against
+// 30, at 128^3 90 against 96.  PBiCG, whose sweeps run without the loads ahead,
+// wants more threads on large meshes: DILU at 64^3 158 against 183, at 128^3 393
+// against 379.
 int default_threads(const spuma_solver_controls* ctl, int64_t n, bool bicg = false)
 {
     if (ctl && ctl->block_threads > 0) return ctl->block_threads;
     if (n <= 50000) return 256;
-    return n <= (bicg ? 1000000 : 3000000) ? 512 : 1024;
+    return bicg && n > 1000000 ? 1024 : 512;
 }
 
 // Blocks of the persistent single-system solver: one per row chunk of
@@ -2206,12 +2448,7 @@ spuma_status launch_batch_kernel(const BatchTable& t, int grid, int threads, int
     return SPUMA_OK;
 }
 
-int batch_kind(int precision)
-{
-    if (precision == SPUMA_MIXED) return KIND_MIXED;
-    if (precision == SPUMA_MIXED_RESTART) return KIND_MIXED_RESTART;
-    return KIND_F64;
-}
+int batch_kind(int precision, int precond) { return precision_kind(precision, precond); }
 
 void fill_controls(SolveArgs& a, const spuma_solver_controls* ctl)
 {
