@@ -254,7 +254,9 @@ spuma_status spuma_precondition(spuma_ldu_t h, int32_t precond, const double* r,
  * < tolerance or after max_outer steps; s = max|r|; inner FP32 PCG on
  * A d = r/s from d = 0 to inner_rel_tol; x += s d.
  * The whole solve is one persistent cooperative kernel (plus the prepare
- * kernels): no host round trip per iteration.  perf is a DEVICE pointer.
+ * kernels): no host round trip per iteration.  A small FP64 DIC system (up to
+ * 38400 rows of at most six entries, 256 levels; block_threads 0) is solved
+ * by one thread-block cluster instead.  perf is a DEVICE pointer.
  * ---------------------------------------------------------------------- */
 spuma_status spuma_pcg_solve(spuma_ldu_t h, const double* diag, const double* upper,
                              const double* b, double* x, const spuma_solver_controls* ctl,
@@ -501,8 +503,9 @@ int32_t spuma_tune_cache_store(const char* path, const char* signature, int32_t 
  * the last host-side error of the calling thread.  spuma_launch_count: the
  * number of kernels this library has launched in the process (a counter on
  * the host, for benchmarks).  spuma_set_barrier_timeout_ns: time limit of
- * every device-side grid-barrier wait in later launches (default 2 s); a test
- * sets it to 0 to check that an expired wait returns
+ * every device-side grid-barrier wait in later launches (default 2 s; a
+ * cluster's hardware barriers have none, so 0 also keeps small systems on
+ * the grid); a test sets it to 0 to check that an expired wait returns
  * SPUMA_ERR_DEVICE_TIMEOUT instead of hanging.
  * ---------------------------------------------------------------------- */
 /* spuma_read_phase_clocks: when the environment variable SPUMA_PHASE_CLOCKS

@@ -120,7 +120,7 @@ struct Group {
     int nblocks;           // blocks in the group
     int bid;               // this block's index in the group
     unsigned long long timeout_ns;
-    static constexpr bool wide = false;
+    static constexpr bool wide = false, cluster = false;
 };
 // A group of blocks of at most 512 threads, whose kernels have 128 registers
 // per thread: their solver phases keep one round of loads ahead.

@@ -475,8 +475,8 @@ __device__ __forceinline__ void vprod(A& acc, double2 x, double2 y)
 // 1422.
 // Asymmetric: row u's lower entry of face f holds lower_f (A) and upper_f
 // (A^T), row l's upper entry upper_f (A) and lower_f (A^T).
-template <bool ASYM>
-__device__ bool phase_gather(const SolveArgs& a, const Group& g)
+template <bool ASYM, class GR>
+__device__ bool phase_gather(const SolveArgs& a, const GR& g)
 {
     constexpr int G = 6;
     RowIter it = rows_of(g);
@@ -588,8 +588,8 @@ __device__ __forceinline__ void scale_entries(double rd, const double* x, double
 // DIC pivots level by level: p_i = d_i - sum_{lower entries} (a a)/p_col,
 // then rD = 1/p and the sweep coefficients rD_row * a (+ FP32 copies).
 // Diagonal: rD = 1/d.
-template <bool ASYM>
-__device__ bool phase_factor(const SolveArgs& a, const Group& g)
+template <bool ASYM, class GR>
+__device__ bool phase_factor(const SolveArgs& a, const GR& g)
 {
     RowIter it = rows_of(g);
     const bool dilu = ASYM && a.precond == SPUMA_PRECOND_DILU, dic = !ASYM && a.precond == SPUMA_PRECOND_DIC;
@@ -1575,7 +1575,8 @@ __device__ bool solve_mixed_eisenstat(const SolveArgs& a, const GR& g, double nf
 
 // x = x_orig (or 0), b = b_orig in internal order; q = A x; r = b - q;
 // normFactor = sum(|q - s xbar| + |b - s xbar|) + 1e-20; returns res0 and nfac.
-__device__ bool phase_init(const SolveArgs& a, const Group& g, double* nfac, double* res0)
+template <class GR>
+__device__ bool phase_init(const SolveArgs& a, const GR& g, double* nfac, double* res0)
 {
     RowIter it = rows_of(g);
     const Mat<double> A = mat_of<double>(a);
@@ -1981,6 +1982,10 @@ __device__ bool solve_pbicg(const SolveArgs& a, const GR& g, double nfac, double
 
 enum SolveKind { KIND_SETUP = 0, KIND_F64 = 1, KIND_MIXED = 2, KIND_MIXED_RESTART = 3, KIND_PBICG = 4, KIND_MIXED_DIC = 5 };
 
+}  // namespace spuma
+#include "small.cuh"
+namespace spuma {
+
 // TRUE_INLINE: the report's true residual is computed inside the launch
 // (batched launches); the single-system solver leaves it to the two small
 // kernels that follow it on the stream (k_true_residual_*), so that its own
@@ -2039,10 +2044,16 @@ __device__ void run_system(const SolveArgs& a, const GR& g)
                     ok = solve_mixed_restart(a, g, nfac, pf);
                 } else {
                     Vecs<double> v{a.x, a.r, a.w, a.p, a.q};
-                    double res;
+                    double res = res0;
                     int sing = 0;
-                    int n_it = pcg_loop<double>(a, mat_of<double>(a), v, nfac, res0, a.tol, a.rel_tol, a.max_iter,
+                    int n_it;
+                    if constexpr (GR::cluster) {
+                        ok = cluster_all_ok(g);
+                        n_it = ok ? small_pcg(a, g, nfac, res0, &res, &sing) : -1;
+                    } else {
+                        n_it = pcg_loop<double>(a, mat_of<double>(a), v, nfac, res0, a.tol, a.rel_tol, a.max_iter,
                                                 a.min_iter, &res, &sing, g);
+                    }
                     ok = n_it >= 0;
                     pf.initial_residual = res0;
                     pf.final_residual = res;
@@ -2092,6 +2103,19 @@ __global__ void __launch_bounds__(MAXT, 1) k_solve(SolveArgs a, unsigned long lo
     g.bid = (int)blockIdx.x;
     g.timeout_ns = timeout_ns;
     run_system<KIND, false>(a, g);
+}
+
+// The FP64 DIC solve of a small system: one cluster or one block (small.cuh).
+template <class GR>
+__global__ void __launch_bounds__(kSmallThreads, 1) k_solve_small(SolveArgs a)
+{
+    GR g;
+    g.word = nullptr;
+    g.status = a.status;
+    g.nblocks = (int)gridDim.x;
+    g.bid = (int)blockIdx.x;
+    g.timeout_ns = 0;
+    run_system<KIND_F64, false>(a, g);
 }
 
 // The single-system solver's true residual, after it on the stream: per-block
@@ -2401,6 +2425,87 @@ int tail_level(spuma_ldu_t h, int threads)
     return (h->nlev - t >= 2) ? t : h->nlev;
 }
 
+// The report's true residual (the solver's x in internal order is still in the
+// workspace).
+static spuma_status launch_true_residual(spuma_ldu_t h, const SolveArgs& b, int kind, cudaStream_t s)
+{
+    const int tg = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)h->n + 255) / 256, (int64_t)h->num_sms * 8));
+    k_true_residual_part<<<tg, 256, 0, s>>>(b, kind == KIND_PBICG ? 1 : 0);
+    k_true_residual_final<<<1, 32, 0, s>>>(b, tg);
+    count_launch(2);
+    SPUMA_CUDA(cudaGetLastError());
+    return SPUMA_OK;
+}
+
+// Blocks of the cluster that solves h's FP64 DIC systems (small.cuh), 0 when the
+// grid solver takes them: rows of more than six entries, more levels than the
+// table holds, or more rows than the blocks hold; and with a time limit of zero,
+// which asks for waits that run out (the cluster's hardware barrier has none).
+static int small_cluster(spuma_ldu_t h)
+{
+    if (barrier_timeout_ns() == 0) return 0;
+    if (h->ell_w < 1 || h->ell_w > 6 || h->nlev > kSmallLevels || h->n > kSmallMaxRows) return 0;
+    return h->n <= kSmallOneBlock ? 1 : kSmallMaxCluster;
+}
+
+static const void* small_kernel(int G)
+{
+    return G > 1 ? (const void*)k_solve_small<ClusterGroup> : (const void*)k_solve_small<BlockGroup>;
+}
+
+// Whether a cluster of G blocks with `smem` bytes can run on the current
+// device (asked once per device, size and amount).
+static bool small_fits(int device, int G, size_t smem, cudaLaunchConfig_t& cfg)
+{
+    static std::map<std::pair<int, long long>, bool> known;
+    std::lock_guard<std::mutex> lk(g_occ_mu);
+    const auto key = std::make_pair(device, (long long)smem * 64 + G);
+    auto it = known.find(key);
+    if (it != known.end()) return it->second;
+    int nc = 0;
+    const void* k = small_kernel(G);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)small_smem(kSmallSlots));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&nc, k, &cfg);
+    if (e != cudaSuccess) cudaGetLastError();
+    return known[key] = e == cudaSuccess && nc > 0;
+}
+
+// Launches the solve on a cluster; false when the grid solver must take it.
+static bool launch_small(spuma_ldu_t h, const SolveArgs& a, cudaStream_t s, spuma_status* st)
+{
+    const int G = small_cluster(h);
+    if (G == 0) return false;
+    const int nslot = ((h->n + 31) / 32 + G - 1) / G * 32;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(G);
+    cfg.blockDim = dim3(kSmallThreads);
+    cfg.dynamicSmemBytes = small_smem(nslot);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = G;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (!small_fits(h->device, G, cfg.dynamicSmemBytes, cfg)) return false;
+    auto run = [&]() -> spuma_status {
+        SPUMA_CUDA(cudaMemsetAsync(h->at<char>(h->L.bar), 0, h->L.status + 256 - h->L.bar, s));
+        SolveArgs b = a;
+        if (getenv("SPUMA_PHASE_CLOCKS")) {
+            b.phase_clk = h->at<long long>(h->L.clk);
+            SPUMA_CUDA(cudaMemsetAsync(b.phase_clk, 0, 8 * 256, s));
+        }
+        void* args[] = {(void*)&b};
+        SPUMA_CUDA(cudaLaunchKernelExC(&cfg, small_kernel(G), args));
+        count_launch();
+        return launch_true_residual(h, b, KIND_F64, s);
+    };
+    *st = run();
+    return true;
+}
+
 spuma_status launch_solve(spuma_ldu_t h, const SolveArgs& a, int threads, cudaStream_t s)
 {
     if (threads < 32 || threads > 1024 || threads % 32) {
@@ -2428,15 +2533,7 @@ spuma_status launch_solve(spuma_ldu_t h, const SolveArgs& a, int threads, cudaSt
     void* args[] = {(void*)&b, (void*)&tns};
     SPUMA_CUDA(cudaLaunchCooperativeKernel(solve_kernel(kind, threads), grid, threads, args, 0, s));
     count_launch();
-    if (b.mode == MODE_SOLVE) {
-        // the report's true residual (the solver's x in internal order is still in the workspace)
-        const int tg = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)h->n + 255) / 256, (int64_t)h->num_sms * 8));
-        k_true_residual_part<<<tg, 256, 0, s>>>(b, kind == KIND_PBICG ? 1 : 0);
-        k_true_residual_final<<<1, 32, 0, s>>>(b, tg);
-        count_launch(2);
-        SPUMA_CUDA(cudaGetLastError());
-    }
-    return SPUMA_OK;
+    return b.mode == MODE_SOLVE ? launch_true_residual(h, b, kind, s) : SPUMA_OK;
 }
 
 spuma_status launch_batch_kernel(const BatchTable& t, int grid, int threads, int kind, cudaStream_t s)
@@ -2508,7 +2605,9 @@ spuma_status pcg_solve_internal(spuma_ldu_t h, const double* diag, const double*
     a.b_orig = b;
     a.x_orig = x;
     a.perf = perf;
-    spuma_status st = launch_solve(h, a, default_threads(ctl, h->n), s);
+    spuma_status st = SPUMA_OK;
+    if (ctl->block_threads != 0 || kind_of(a) != KIND_F64 || a.precond != SPUMA_PRECOND_DIC || !launch_small(h, a, s, &st))
+        st = launch_solve(h, a, default_threads(ctl, h->n), s);
     if (st == SPUMA_OK) h->prepared_precond = ctl->precond;
     return st;
 }
