@@ -55,9 +55,9 @@ constexpr int kGamgPostSweeps = 2;
 // FP64 pipe takes as long for a level of 700 cells (40 us, Gauss-Seidel) as the
 // whole grid with its barriers for one of 20 thousand; per V-cycle at 64^3
 // (Richardson) / 128^3 (Gauss-Seidel), limit 2048: 288 / 1370 us, 768: 270 /
-// 1321, 300: 261 / 1306, 100: 265 / 1310.
+// 1321, 300: 261 / 1306, 100: 265 / 1310.  256: what two rows per team hold.
 constexpr int kGamgThreads = 512;
-constexpr int kGamgSmall = 300;
+constexpr int kGamgSmall = 256;
 constexpr double kGamgCoarseRelTol = 1e-8;
 enum GamgSlot { GS_A = 0, GS_B = 1, GS_C = 2, GS_D = 3 };   // reduction slots
 
@@ -286,10 +286,8 @@ __device__ __forceinline__ void lvl0_rows(const GamgLvl0& z, const int* cols, co
 #pragma unroll
             for (int j = 0; j < 6; j++) c[j] = j < z.ell_w ? __ldcs(cols + (size_t)j * z.n + p) : -1;
         };
-        int cur[6];
-        if (first < n) load(cur, first);
-        for (int p = first; p < n; p += stride) {
-            int nxt[6];
+        // two sets of indices take turns (a copy would wait for the loads)
+        auto row = [&](int (&cur)[6], int (&nxt)[6], int p) {
             const int pn = p + stride;
             if (pn < n) load(nxt, pn);
             double g6[6];
@@ -302,8 +300,12 @@ __device__ __forceinline__ void lvl0_rows(const GamgLvl0& z, const int* cols, co
             for (int j = 0; j < 6; j++)
                 if (cur[j] >= 0) y = __fma_rn(__ldcs(z.Ea + (size_t)j * z.n + p), g6[j], y);
             body(p, y, xp, u, w);
-#pragma unroll
-            for (int j = 0; j < 6; j++) cur[j] = nxt[j];
+        };
+        int ca[6], cb[6];
+        if (first < n) load(ca, first);
+        for (int p = first; p < n; p += 2 * stride) {
+            row(ca, cb, p);
+            if (p + stride < n) row(cb, ca, p + stride);
         }
         return;
     }
@@ -314,35 +316,68 @@ __device__ __forceinline__ void lvl0_rows(const GamgLvl0& z, const int* cols, co
     }
 }
 
+// A team's sums of RT rows from its lanes' parts, in a fixed order: row t in lane
+// t (t < RT); returns the lane's row.
+template <int RT>
+__device__ __forceinline__ int team_add(const double (&s)[RT], int t, double& r)
+{
+    if constexpr (RT == 1) {
+        r = __dadd_rn(s[0], __shfl_xor_sync(0xffffffffu, s[0], 1));
+        r = __dadd_rn(r, __shfl_xor_sync(0xffffffffu, r, 2));
+        return 0;
+    } else if constexpr (RT == 2) {
+        const bool odd = t & 1;
+        r = __dadd_rn(odd ? s[1] : s[0], __shfl_xor_sync(0xffffffffu, odd ? s[0] : s[1], 1));
+        r = __dadd_rn(r, __shfl_xor_sync(0xffffffffu, r, 2));
+        return t & 1;
+    } else {
+        const bool odd = t & 1, high = t & 2;   // rows of the lane's parity first, then its half
+        const double lo = __dadd_rn(odd ? s[1] : s[0], __shfl_xor_sync(0xffffffffu, odd ? s[0] : s[1], 1));
+        const double hi = __dadd_rn(odd ? s[3] : s[2], __shfl_xor_sync(0xffffffffu, odd ? s[2] : s[3], 1));
+        r = __dadd_rn(high ? hi : lo, __shfl_xor_sync(0xffffffffu, high ? lo : hi, 2));
+        return t;
+    }
+}
+
 // Coarse rows [c0, end) of one block by teams of four lanes: body(i, sum over
 // the row's entries, the first cnt_i of them when cnt is given, of val_e
 // v[col_e]), called on one lane per row.  A team's lanes take every fourth
 // entry (neighbouring lanes read neighbouring entries) and add up in a fixed
 // order.  RT rows per team: 4 on levels that fill the block, where the lanes
 // then hold one finished row each (three adds for four rows, and the body runs
-// on every lane); 1 below, for the shorter chain.  A warp's FP64 instruction
-// takes its quadrant's pipe for 64 cycles however many lanes are live: a
-// thread per row pays for the longest of 32 rows (20 to 25 entries against 9
-// to 15 on average), one entry after the other.
+// on every lane), fewer below for the shorter chain.  The next rows' extents
+// load beside a row's entries.  A warp's FP64 instruction takes its quadrant's
+// pipe for 64 cycles however many lanes are live: a thread per row pays for the
+// longest of 32 rows (20 to 25 entries against 9 to 15 on average), one entry
+// after the other.
 template <int RT, class Body>
 __device__ __forceinline__ void team_rows_t(const int* rptr, const int* cnt, const int* col, const double* val,
                                             const double* v, int c0, int end, Body body)
 {
-    static_assert(RT == 1 || RT == 4, "rows per team");
-    constexpr int G = RT == 1 ? 4 : 2;      // entries per lane and load group
+    static_assert(RT == 1 || RT == 2 || RT == 4, "rows per team");
+    constexpr int G = RT == 4 ? 2 : 4;      // entries per lane and load group
     const int t = (int)threadIdx.x & 3, per = ((int)blockDim.x >> 2) * RT;
+    int b0[RT], b1[RT];
+    auto extents = [&](int i0) {
+#pragma unroll
+        for (int k = 0; k < RT; k++) {
+            const bool ok = i0 + k < end;
+            b0[k] = ok ? __ldg(rptr + i0 + k) : 0;
+            b1[k] = ok ? (cnt ? __ldg(cnt + i0 + k) : __ldg(rptr + i0 + k + 1)) : 0;
+        }
+    };
+    extents(c0 + ((int)threadIdx.x >> 2) * RT);
     for (int base = c0; base < end; base += per) {
         const int i0 = base + ((int)threadIdx.x >> 2) * RT;
         double s[RT];
         int e[RT], e1[RT];
 #pragma unroll
         for (int k = 0; k < RT; k++) {
-            const bool ok = i0 + k < end;
-            const int b = ok ? rptr[i0 + k] : 0;
-            e1[k] = ok ? (cnt ? b + cnt[i0 + k] : rptr[i0 + k + 1]) : 0;
-            e[k] = b + t;
+            e[k] = b0[k] + t;
+            e1[k] = cnt ? b0[k] + b1[k] : b1[k];
             s[k] = 0.0;
         }
+        bool ahead = true;
         for (;;) {
             bool more = false;
 #pragma unroll
@@ -358,6 +393,10 @@ __device__ __forceinline__ void team_rows_t(const int* rptr, const int* cnt, con
                     c[k][j] = ok ? __ldg(col + e[k] + 4 * j) : -1;
                     a[k][j] = ok ? val[e[k] + 4 * j] : 0.0;
                 }
+            if (ahead) {
+                extents(i0 + per);
+                ahead = false;
+            }
 #pragma unroll
             for (int k = 0; k < RT; k++)
 #pragma unroll
@@ -370,41 +409,60 @@ __device__ __forceinline__ void team_rows_t(const int* rptr, const int* cnt, con
                 e[k] += 4 * G;
             }
         }
+        if (ahead) extents(i0 + per);
         __syncwarp();
-        if (RT == 1) {
-            double r = s[0];
-            r = __dadd_rn(r, __shfl_xor_sync(0xffffffffu, r, 1));
-            r = __dadd_rn(r, __shfl_xor_sync(0xffffffffu, r, 2));
-            if (t == 0 && i0 < end) body(i0, r);
-        } else {
-            // lane t ends with row i0 + t: rows of its parity first, then its half
-            const bool odd = t & 1, high = t & 2;
-            double lo = odd ? s[1 % RT] : s[0], lo_out = odd ? s[0] : s[1 % RT];
-            double hi = odd ? s[3 % RT] : s[2 % RT], hi_out = odd ? s[2 % RT] : s[3 % RT];
-            lo = __dadd_rn(lo, __shfl_xor_sync(0xffffffffu, lo_out, 1));
-            hi = __dadd_rn(hi, __shfl_xor_sync(0xffffffffu, hi_out, 1));
-            const double keep = high ? hi : lo, out = high ? lo : hi;
-            const double r = __dadd_rn(keep, __shfl_xor_sync(0xffffffffu, out, 2));
-            if (i0 + t < end) body(i0 + t, r);
-        }
+        double r;
+        const int m = team_add<RT>(s, t, r);
+        if (t < RT && i0 + m < end) body(i0 + m, r);
     }
 }
 template <class Body>
 __device__ __forceinline__ void team_rows(const GamgLevel& L, const int* cnt, const int* col, const double* v,
                                           const Exec& x, Body body)
 {
-    if (x.end - x.c0 > (int)blockDim.x / 2)
+    const int rows = x.end - x.c0, teams = (int)blockDim.x >> 2;
+    if (rows > 2 * teams)
         team_rows_t<4>(L.rptr, cnt, col, L.rval, v, x.c0, x.end, body);
+    else if (rows > teams)
+        team_rows_t<2>(L.rptr, cnt, col, L.rval, v, x.c0, x.end, body);
     else
         team_rows_t<1>(L.rptr, cnt, col, L.rval, v, x.c0, x.end, body);
 }
 
-// s - sum over level 0's lower entries (face order) of a_f y_col, one FMA each
-// (the two-stage Gauss-Seidel's second stage).
-__device__ __forceinline__ double lvl0_lower_sweep(const GamgLvl0& z, const double* y, int i, double s)
+// Level 0's lower sweep over rows first, first + stride, ... below n (the
+// two-stage Gauss-Seidel's second stage): body(i, q_i - sum over the row's
+// lower entries, in face order, of a_f y_col, one FMA each).  Entries in groups
+// of 6, the next row's extents loaded beside them.
+template <class Body>
+__device__ __forceinline__ void lvl0_lower_rows(const GamgLvl0& z, const double* y, const double* q, int first,
+                                                int stride, int n, Body body)
 {
-    for (int e = z.Lptr[i]; e < z.Lptr[i + 1]; e++) s = __fma_rn(-z.La[e], y[z.Lcol[e]], s);
-    return s;
+    int n0 = first < n ? __ldcs(z.Lptr + first) : 0, n1 = first < n ? __ldcs(z.Lptr + first + 1) : 0;
+    for (int p = first; p < n; p += stride) {
+        const int e0 = n0, e1 = n1, pn = p + stride;
+        double s = q[p];
+        for (int off = e0;; off += 6) {
+            int c[6];
+            double a[6], x[6];
+#pragma unroll
+            for (int j = 0; j < 6; j++) {
+                const bool ok = off + j < e1;
+                c[j] = ok ? __ldcs(z.Lcol + off + j) : -1;
+                a[j] = ok ? __ldcs(z.La + off + j) : 0.0;
+            }
+            if (off == e0) {
+                n0 = pn < n ? __ldcs(z.Lptr + pn) : 0;
+                n1 = pn < n ? __ldcs(z.Lptr + pn + 1) : 0;
+            }
+#pragma unroll
+            for (int j = 0; j < 6; j++) x[j] = c[j] >= 0 ? y[c[j]] : 0.0;
+#pragma unroll
+            for (int j = 0; j < 6; j++)
+                if (c[j] >= 0) s = __fma_rn(-a[j], x[j], s);
+            if (off + 6 >= e1) break;
+        }
+        body(p, s);
+    }
 }
 
 // Level 0's coefficients in internal order (per solve): the CSR entries, the
@@ -661,6 +719,160 @@ __device__ bool gamg_coarsest(const GamgArgs& a, const Group& g, const CoarseDen
     return exec_sync(x, g);
 }
 
+// Levels whose rows fill no more than one pass of the block's teams (RT rows
+// each) keep everything a row needs in its team's registers for the whole
+// level: the first 16 entries, their columns and aggregates, r, 1/d and the
+// rest; and the next level's are loaded before the level's last barrier, so
+// that between two barriers only the gathers, the sums and a store remain.
+// Warp 0 of a grid block takes no rows (the fence of its barrier arrival would
+// wait for the loads ahead).  Per V-cycle, against every step reading its lists: 64^3
+// Richardson 259 -> 249 us, 128^3 two-stage Gauss-Seidel 1320 -> 1298 us.
+template <int RT>
+struct TeamLevel {
+    int b[RT], e1[RT], lo[RT];          // entry ranges, lower entries
+    int cc[RT][4], ca[RT][4];           // columns and their aggregates
+    double v[RT][4];
+    int row, agg;                       // the lane's own row (-1: none)
+    double r, w, d;
+};
+
+// The solo levels of the first block (no service warp, block barriers).
+template <int RT, bool SOLO>
+struct TeamLevels {
+    const GamgArgs& a;
+    const Group& g;
+    int t, team, teams;
+
+    __device__ __forceinline__ TeamLevels(const GamgArgs& a_, const Group& g_) : a(a_), g(g_)
+    {
+        const int svc = SOLO ? 0 : kWarp, id = (int)threadIdx.x - svc;
+        t = (int)threadIdx.x & 3;
+        team = id >> 2;                 // negative in the service warp
+        teams = ((int)blockDim.x - svc) >> 2;
+    }
+    __device__ __forceinline__ void load(int k, TeamLevel<RT>& q) const
+    {
+        const GamgLevel& L = a.lv[k];
+        const Exec x = exec_for(a, k, g, L.n);
+        const int i0 = x.c0 + team * RT;
+#pragma unroll
+        for (int m = 0; m < RT; m++) {
+            const bool ok = team >= 0 && i0 + m < x.end;
+            q.b[m] = ok ? __ldg(L.rptr + i0 + m) : 0;
+            q.e1[m] = ok ? __ldg(L.rptr + i0 + m + 1) : 0;
+            q.lo[m] = ok ? __ldg(L.rlo + i0 + m) : 0;
+        }
+        q.row = team >= 0 && t < RT && i0 + t < x.end ? i0 + t : -1;
+        q.agg = 0;
+        q.r = q.w = q.d = 0.0;
+        if (q.row >= 0) {
+            q.agg = __ldg(L.agg + q.row);
+            q.w = L.wrd[q.row];
+            q.d = L.diag[q.row];
+            q.r = L.r[q.row];
+        }
+#pragma unroll
+        for (int m = 0; m < RT; m++)
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const int e = q.b[m] + t + 4 * j;
+                const bool ok = e < q.e1[m];
+                q.cc[m][j] = ok ? __ldg(L.rcol + e) : -1;
+                q.ca[m][j] = ok ? __ldg(L.cagg + e) : -1;
+                q.v[m][j] = ok ? L.rval[e] : 0.0;
+            }
+    }
+    // Sum over the rows' entries (the lower ones with LOWER) of val_e vec[index_e],
+    // AGG: through the aggregates; the lane's own row's sum.
+    template <bool AGG, bool LOWER>
+    __device__ __forceinline__ double sum(const GamgLevel& L, const TeamLevel<RT>& q, const double* vec) const
+    {
+        double x[RT][4], s[RT], r;
+#pragma unroll
+        for (int m = 0; m < RT; m++)
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const int c = AGG ? q.ca[m][j] : q.cc[m][j];
+                x[m][j] = c >= 0 && (!LOWER || t + 4 * j < q.lo[m]) ? vec[c] : 0.0;
+            }
+#pragma unroll
+        for (int m = 0; m < RT; m++) {
+            s[m] = 0.0;
+            const int end = LOWER ? q.b[m] + q.lo[m] : q.e1[m];
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                if (q.b[m] + t + 4 * j < end) s[m] = __fma_rn(q.v[m][j], x[m][j], s[m]);
+            for (int e = q.b[m] + t + 16; e < end; e += 4)   // rows of more than 16 entries
+                s[m] = __fma_rn(L.rval[e], vec[__ldg((AGG ? L.cagg : L.rcol) + e)], s[m]);
+        }
+        __syncwarp();
+        team_add<RT>(s, t, r);
+        return r;
+    }
+    __device__ __forceinline__ bool sync() const
+    {
+        if constexpr (SOLO) {
+            __syncthreads();
+            return true;
+        }
+        return group_sync(g);
+    }
+
+    // Levels from .. to (descending), all of this kind.
+    __device__ bool up(int from, int to, GamgClock& ck) const
+    {
+        TeamLevel<RT> q;
+        load(from, q);
+        for (int k = from; k >= to; k--) {
+            const GamgLevel& L = a.lv[k];
+            const double* ec = a.lv[k + 1].e;
+            const bool own = q.row >= 0;
+            const double s0 = sum<true, false>(L, q, ec);
+            const double ei = own ? ec[q.agg] : 0.0;
+            const double ae = __fma_rn(q.d, ei, s0);
+            double v[2] = {own ? __dmul_rn(ei, q.r) : 0.0, own ? __dmul_rn(ei, ae) : 0.0};
+            Exec x{0, 0, 0, 0, !SOLO, true};
+            if (!exec_sum<2>(x, v, a, GS_A, g)) return false;
+            const double sc = v[1] > 0.0 ? v[0] / v[1] : 1.0;
+            double qi = __fma_rn(-sc, ae, q.r), yi, e0 = __dmul_rn(sc, ei);
+            if (a.smoother == 1) {
+                for (int m = 0; m < kGamgPostSweeps; m++) {
+                    if (m > 0) qi = __dsub_rn(q.r, __fma_rn(q.d, e0, sum<false, false>(L, q, L.e)));
+                    yi = __dmul_rn(q.w, qi);
+                    if (own) L.y[q.row] = yi;
+                    if (!sync()) return false;
+                    e0 = __fma_rn(q.w, __dsub_rn(qi, sum<false, true>(L, q, L.y)), e0);
+                    if (own) L.e[q.row] = e0;
+                    if (m == kGamgPostSweeps - 1 && k > to) load(k - 1, q);
+                    if (!sync()) return false;
+                }
+            } else {
+                yi = __fma_rn(q.w, qi, e0);
+                if (own) L.y[q.row] = yi;
+                if (!sync()) return false;
+                const double ay = __fma_rn(q.d, yi, sum<false, false>(L, q, L.y));
+                if (own) L.e[q.row] = __fma_rn(q.w, __dsub_rn(q.r, ay), yi);
+                if (k > to) load(k - 1, q);
+                if (!sync()) return false;
+            }
+            ck.lap(64 + k);
+        }
+        return true;
+    }
+};
+
+// Rows per team of level k's kind: 1 or 2 when its rows fit one pass, else 0
+// (level 0 has passes of its own).
+__device__ __forceinline__ int team_kind(const GamgArgs& a, int k, const Group& g)
+{
+    if (k == 0) return 0;
+    const int n = a.lv[k].n, bs = (int)blockDim.x;
+    const bool solo = k >= a.small_from;
+    const int rows = solo ? n : ((n + g.nblocks - 1) / g.nblocks + 31) & ~31;
+    const int teams = (solo ? bs : bs - kWarp) >> 2;
+    return rows <= teams ? 1 : rows <= 2 * teams ? 2 : 0;
+}
+
 // e_0 = V(0, r_0), with r_0 = a.res; the last smoothing sweep of level 0 also
 // adds e_0 to x (the outer update, fused).
 __device__ bool gamg_vcycle(const GamgArgs& a, const Group& g, const CoarseDense& D, GamgClock& ck)
@@ -696,6 +908,21 @@ __device__ bool gamg_vcycle(const GamgArgs& a, const Group& g, const CoarseDense
         const double* ec = a.lv[k + 1].e;
         const double* dg = L.diag;
         if (k + 1 == a.small_from && !group_sync(g)) return false;   // the first block's levels are done
+        if (const int kind = team_kind(a, k, g)) {
+            // the run of levels of this kind
+            const bool solo = k >= a.small_from;
+            int to = k;
+            while (to > 0 && to != a.small_from && team_kind(a, to - 1, g) == kind) to--;
+            bool ok = true;
+            if (solo) {
+                if (g.bid == 0) ok = kind == 1 ? TeamLevels<1, true>(a, g).up(k, to, ck) : TeamLevels<2, true>(a, g).up(k, to, ck);
+            } else {
+                ok = kind == 1 ? TeamLevels<1, false>(a, g).up(k, to, ck) : TeamLevels<2, false>(a, g).up(k, to, ck);
+            }
+            if (!ok) return false;
+            k = to;
+            continue;
+        }
         const Exec x = exec_for(a, k, g, L.n);
         // q = A P e_c, (e.r), (e.A e)
         double v[2] = {0.0, 0.0};
@@ -752,12 +979,11 @@ __device__ bool gamg_vcycle(const GamgArgs& a, const Group& g, const CoarseDense
                 if (x.active) {
                     if (k == 0) {
                         const bool fold = s == kGamgPostSweeps - 1;   // x += e_0 here
-                        for (int i = x.first; i < x.end; i += x.stride) {
-                            const double si = lvl0_lower_sweep(a.z, L.y, i, L.q[i]);
+                        lvl0_lower_rows(a.z, L.y, L.q, x.first, x.stride, x.end, [&](int i, double si) {
                             const double ei = __fma_rn(L.wrd[i], si, L.e[i]);
                             L.e[i] = ei;
                             if (fold) a.x[i] = __dadd_rn(a.x[i], ei);
-                        }
+                        });
                     } else {
                         team_rows(L, L.rlo, L.rcol, L.y, x, [&](int i, double ly) {
                             L.e[i] = __fma_rn(L.wrd[i], __dsub_rn(L.q[i], ly), L.e[i]);
@@ -794,8 +1020,19 @@ __device__ bool gamg_vcycle(const GamgArgs& a, const Group& g, const CoarseDense
     return true;
 }
 
-__global__ void __launch_bounds__(kGamgThreads, 1) k_gamg(GamgArgs a, unsigned long long timeout_ns)
+__global__ void __launch_bounds__(kGamgThreads, 1) k_gamg(GamgArgs args, unsigned long long timeout_ns)
 {
+    // the levels' descriptors in shared memory: every barrier's acquire drops the
+    // L1, and a step would begin with a trip to L2 for its pointers
+    __shared__ GamgLevel levels[kGamgMaxLevels];
+    __shared__ GamgArgs a;
+    for (int i = threadIdx.x; i < (int)(args.nlev * sizeof(GamgLevel) / 8); i += blockDim.x)
+        reinterpret_cast<unsigned long long*>(levels)[i] = reinterpret_cast<const unsigned long long*>(args.lv)[i];
+    if (threadIdx.x == 0) {
+        a = args;
+        a.lv = levels;
+    }
+    __syncthreads();
     Group g{reinterpret_cast<unsigned long long*>(a.status + DS_BARRIER), a.status, (int)gridDim.x, (int)blockIdx.x, timeout_ns};
     spuma_solver_perf pf{};
     pf.n_levels = a.nlev;

@@ -1,8 +1,8 @@
 """GPU: the solver kernels that a solve is routed to by its size and shape, each
 at the ends of its range, against the oracle's PCG at the same iteration count:
 one block (small systems), a cluster of blocks, the grid with loads ahead (up
-to 512 threads) and without (1024), FP64 and mixed; and PBiCG on rows wider
-than its entry groups."""
+to 512 threads) and without (1024), FP64 and mixed; PBiCG on rows wider than
+its entry groups; and GAMG by the sizes of its levels."""
 import numpy as np
 import pytest
 import torch
@@ -110,3 +110,21 @@ def test_pbicg_wide_rows(threads):
     assert p["converged"] == 1 and p["status"] == 0
     xo, _ = oracle.pbicg(lo, ua, d, lower, upper, c.b, precond=3, tol=0.0, max_iter=p["n_iter"])
     assert np.linalg.norm(x.cpu().numpy() - xo) <= 1e-9 * np.linalg.norm(xo)
+
+
+# levels of the sizes where the rows per team change: 240 and 112 cells on the first block (two rows, one); 12560 on the
+# grid (one) and 17770 (two: 128 rows per block, 124 teams)
+@pytest.mark.parametrize("n", [(8, 8, 8), (30, 30, 30), (34, 34, 33)])
+@pytest.mark.parametrize("smoother,name", [(0, "richardson"), (1, "gs2")])
+def test_gamg_level_sizes(n, smoother, name):
+    from oracle import gamg
+    from paper_2512_22215_gb300 import GamgSolver, SolverControls
+    c = case(n, jitter=0.2, permute=True, seed=108, lognormal=True)
+    m = c.mesh
+    uo, do = assemble_oracle(c)
+    w = np.linalg.norm(m.sf, axis=1)
+    S = GamgSolver(mesh_of(c, centres=True), dev(w), smoother=smoother)
+    x, p = S.solve(dev(do), dev(uo), dev(c.b), None, SolverControls(tolerance=0.0, max_iter=3))
+    assert p["n_iter"] == 3 and p["status"] == 0
+    xo, _, _ = gamg.gamg(m.lower, m.upper_addr, do, uo, c.b, w, tol=0.0, max_iter=3, smoother=name)
+    assert np.linalg.norm(x.cpu().numpy() - xo) <= 1e-8 * np.linalg.norm(xo)
