@@ -7,17 +7,20 @@
 // cycles, about 9 of them, a __dsqrt_rn 671.  Here the reciprocal (square
 // root) starts from a float-float value of about 44 bits, made on the FP32 and
 // integer pipes from the operand's bits, and one FP64 Newton step brings it
-// within half a unit of 1/b (to 2^-34 of a unit).  Markstein's theorem (P. W.
-// Markstein, "Computation of elementary functions on the IBM RISC System/6000
-// processor", IBM J. Res. Dev. 34, 1990) then gives the quotient: with y = 1/b
-// rounded, b's mantissa not all ones, and q next to a/b, RN(q + RN(a - b q) y)
-// = RN(a/b).  A reciprocal takes 3 FP64 instructions, each quotient by the
-// same divisor 3 more; a square root with its reciprocal takes 8.  Operands
-// outside the stated ranges (zeros, infinities, NaN, very large or small
-// values, all-ones divisors) take the built-in operations.  Checked on the CPU
-// against IEEE division and square root: 60 million operand pairs, a third of
-// them next to the ends of the mantissa, no difference.  Times: at the face
-// kernels that use them.
+// within half a unit of 1/b (to 2^-34 of a unit).  The quotient follows
+// Markstein (P. W. Markstein, "Computation of elementary functions on the IBM
+// RISC System/6000 processor", IBM J. Res. Dev. 34, 1990): with y = 1/b rounded
+// and q next to a/b, RN(q + RN(a - b q) y) = RN(a/b).  The slack of y against
+// that theorem: the sum misses a/b by |a/b - q| |b y - 1|, and a/b (b in [1, 2))
+// stays 2^-53/b units from a midpoint, so a y within 1/2 + s units serves every
+// b with b^2 (1 + 2 s) < 4: for s = 2^-34 all but the b within 2^-33 of 2.  There,
+// b = 2 - k 2^-52, 1/b lies k^2 2^-54 units from a multiple of half a unit, so y is
+// 1/b rounded from k = 2^10 on; divisor_ok refuses the k up to 2^12 (a/b =
+// 0x1.6666666666663p+0 / 0x1.ffffffffffffbp+0 fails without).  A reciprocal takes
+// 3 FP64 instructions, each quotient by the same divisor 3 more; a square root
+// with its reciprocal takes 8.  Operands outside the stated ranges (zeros,
+// infinities, NaN, very large or small values, those divisors) take the built-in
+// operations.  Times: at the face kernels that use them.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -28,11 +31,12 @@ __device__ __forceinline__ int exp_bits(double v) { return (__double2hiint(v) >>
 // remainders a - b q, stay normal
 __device__ __forceinline__ bool mid_range(double v) { return (unsigned)(exp_bits(v) - (1023 - 300)) < 600u; }
 
-// A divisor for the forms below: positive, mid_range, mantissa not all ones.
+// A divisor for the forms below: positive, mid_range, mantissa not among the 2^12
+// below all ones.
 __device__ __forceinline__ bool divisor_ok(double b)
 {
     const int hi = __double2hiint(b);
-    return hi > 0 && mid_range(b) && !((hi & 0xfffff) == 0xfffff && __double2loint(b) == -1);
+    return hi > 0 && mid_range(b) && !((hi & 0xfffff) == 0xfffff && (unsigned)__double2loint(b) >= 0xfffff000u);
 }
 
 // A float's value times 2^e as a double, by its bits (|v| from 2^-126 up; a
