@@ -110,10 +110,13 @@ __device__ __forceinline__ double sqrt_rn(double v, double& inv)
     const double half = __hiloint2double(__double2hiint(y0) - (1 << 20), __double2loint(y0));
     double g = __dmul_rn(v, y0);
     g = __fma_rn(__fma_rn(-g, g, v), half, g);              // within half a unit plus 2^-86
-    const double y1 = __fma_rn(__fma_rn(-g, y0, 1.0), y0, y0);   
+    const double y1 = __fma_rn(__fma_rn(-g, y0, 1.0), y0, y0);
     const double h1 = __hiloint2double(__double2hiint(y1) - (1 << 20), __double2loint(y1));
-    inv = y1;
-    return __fma_rn(__fma_rn(-g, g, v), h1, g);
+    const double root = __fma_rn(__fma_rn(-g, g, v), h1, g);
+    // y1 is 1/g: of use for the root unless this last step moved it (sqrt(v)
+    // within 2^-34 of a unit of a midpoint)
+    inv = __double2loint(root) == __double2loint(g) ? y1 : recip(root);
+    return root;
 }
 
 // |S|, its reciprocal, and whether quotients by |S| may use it.

@@ -48,3 +48,53 @@ def test_hard_quotients(divisors):
     unit = np.zeros((len(a), 3))
     unit[:, 0] = 1.0
     assert np.array_equal(bits(face_coefficients(unit, unit * b[:, None], a)), bits(a / b))
+
+
+def squares_near_midpoints(count):
+    """Doubles v in [1, 4) whose square root lies just above a midpoint m of two doubles: v = m^2 + j 2^-108 or so, j
+    small (m^2 = -j modulo a power of two, solved bit by bit)."""
+    out = []
+    for r in range(-7, -8 * count, -8):
+        for odd in (0, 1):
+            k = 54 + odd
+            x = 1
+            for n in range(3, k):
+                x += ((x * x - r) >> n & 1) << (n - 1)
+            half = 1 << (k - 1)
+            for M in {x % (2 * half), -x % (2 * half), (x + half) % (2 * half), (half - x) % (2 * half)}:
+                V = (M * M - r) >> k
+                if M >> 53 == 1 and V >> 52 == 1:
+                    out.append(math.ldexp(V, odd - 52))
+    return out
+
+
+def test_hard_quotients_by_the_norm():
+    """n.S = (S.d)/|S| next to a midpoint, where |S|^2 has a square root next to one too: what the square root leaves
+    as 1/|S| has to be the reciprocal of the rounded root."""
+    sf, d, num = [], [], []
+    for v in squares_near_midpoints(800):
+        mag = math.sqrt(v)
+        B = int(mag * 2 ** 52)
+        # S = (x, y, 0) with x^2 + y^2 = v as the kernels add it up
+        x = math.nextafter(mag, 0.0)
+        for _ in range(40):
+            y = math.sqrt(v - x * x)
+            if x * x + y * y == v:
+                break
+            x = math.nextafter(x, 0.0)
+        if not B & 1 or x * x + y * y != v:
+            continue
+        for a in hard_numerators(B):
+            for dx in (a / x, math.nextafter(a / x, 0.0), math.nextafter(a / x, 4.0)):
+                if x * dx == a:
+                    sf.append((x, y, 0.0))
+                    d.append(dx)
+                    num.append((a, mag))
+                    break
+    assert len(num) > 1500
+    sf, d, (a, mag) = np.array(sf), np.array(d), np.array(num).T
+    dist = np.zeros_like(sf)
+    dist[:, 0] = d
+    for gamma in (1.0, 1.25, 1.7):
+        want = (gamma * mag) / (a / mag)      # n.S is far above 0.05 |d|
+        assert np.array_equal(bits(face_coefficients(sf, dist, np.full(len(a), gamma))), bits(want))
