@@ -25,7 +25,15 @@
 
 namespace spuma {
 
-enum Slot { SL_A = 0, SL_B = 1, SL_C = 2, SL_D = 3 };
+// Slots of the block partials.  A slot may be written again only after a grid
+// barrier that follows its last read: a block may still be reading when a
+// faster one goes on.  What follows a read without a barrier in between has
+// slots of its own: the initial sums, after which the loops' first sums (SL_A,
+// SL_B; SL_D and SL_DMAX in the restarted form) or the true residual of a system
+// that starts converged come at once, and the true residual, which follows the
+// sums that stopped the loop.
+enum Slot { SL_A = 0, SL_B = 1, SL_D = 2, SL_DMAX = 3, SL_C = 4, SL_INIT = SL_C, SL_TRUE = 6 };
+static_assert(SL_TRUE + 2 <= kSlots, "two partial sums of the true residual");
 
 __device__ __forceinline__ bool converged(double res, double res0, double tol, double rel_tol)
 {
@@ -1273,11 +1281,11 @@ __device__ bool refine_residual(const SolveArgs& a, const Group& g, bool fold, d
         mx[0] = fmax(mx[0], fabs(rr));
     }
     block_reduce_store<1>(acc, a.partials, SL_D, g.bid);
-    block_max_store<1>(mx, a.partials, SL_D + 1, g.bid);
+    block_max_store<1>(mx, a.partials, SL_DMAX, g.bid);
     if (!group_sync(g)) return false;
     double t[1], m[1];
     grid_reduce_read<1>(t, a.partials, SL_D, g.nblocks);
-    grid_reduce_read<1, true>(m, a.partials, SL_D + 1, g.nblocks);
+    grid_reduce_read<1, true>(m, a.partials, SL_DMAX, g.nblocks);
     *ressum = t[0];
     *rmax = m[0];
     return true;
@@ -1610,9 +1618,9 @@ __device__ bool phase_init(const SolveArgs& a, const GR& g, double* nfac, double
         t2[0] += fabs(qq - tt) + fabs(bv - tt);
         t2[1] += fabs(rr);
     }
-    block_reduce_store<2>(t2, a.partials, SL_B, g.bid);
+    block_reduce_store<2>(t2, a.partials, SL_INIT, g.bid);
     if (!group_sync(g)) return false;
-    grid_reduce_read<2>(t2, a.partials, SL_B, g.nblocks);
+    grid_reduce_read<2>(t2, a.partials, SL_INIT, g.nblocks);
     const double sum_r = t2[1];
     *nfac = t2[0] + 1e-20;
     *res0 = sum_r / *nfac;
@@ -1636,10 +1644,10 @@ __device__ bool true_residual(const SolveArgs& a, const Mat<double>& A, const do
         acc[0] = __fma_rn(rr, rr, acc[0]);
         acc[1] = __fma_rn(bv, bv, acc[1]);
     }
-    block_reduce_store<2>(acc, a.partials, SL_A, g.bid);
+    block_reduce_store<2>(acc, a.partials, SL_TRUE, g.bid);
     if (!group_sync(g)) return false;
     double t[2];
-    grid_reduce_read<2>(t, a.partials, SL_A, g.nblocks);
+    grid_reduce_read<2>(t, a.partials, SL_TRUE, g.nblocks);
     *out = t[1] > 0.0 ? __ddiv_rn(__dsqrt_rn(t[0]), __dsqrt_rn(t[1])) : __dsqrt_rn(t[0]);
     return true;
 }
