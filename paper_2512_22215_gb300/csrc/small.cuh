@@ -41,8 +41,18 @@ struct ClusterGroup : Group {
     static constexpr bool cluster = true, several = true;
 };
 
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// The aligned forms want the warp converged, and callers come here out of loops
+// and branches that its lanes leave at different times.
+__device__ __forceinline__ void cluster_arrive()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_barrier()
 {
     cluster_arrive();
@@ -215,7 +225,6 @@ struct SmallSolve {
             lb += W;
             const bool add = some && (!fwd || L == a.nlev - 1);   // top level: w is final going up
             if (lb >= t.y) {
-                __syncwarp();
                 barrier_arrive();
                 arrived = true;
                 L += step;
