@@ -504,8 +504,8 @@ int32_t spuma_tune_cache_store(const char* path, const char* signature, int32_t 
  * number of kernels this library has launched in the process (a counter on
  * the host, for benchmarks).  spuma_set_barrier_timeout_ns: time limit of
  * every device-side grid-barrier wait in later launches (default 2 s; a
- * cluster's hardware barriers have none, so 0 also keeps small systems on
- * the grid); a test sets it to 0 to check that an expired wait returns
+ * cluster's hardware barriers have none, so a limit below 1 ms also keeps
+ * small systems on the grid); a test sets it to 0 to check that an expired wait returns
  * SPUMA_ERR_DEVICE_TIMEOUT instead of hanging.
  * ---------------------------------------------------------------------- */
 /* spuma_read_phase_clocks: when the environment variable SPUMA_PHASE_CLOCKS

@@ -2447,11 +2447,14 @@ static spuma_status launch_true_residual(spuma_ldu_t h, const SolveArgs& b, int 
 
 // Blocks of the cluster that solves h's FP64 DIC systems (small.cuh), 0 when the
 // grid solver takes them: rows of more than six entries, more levels than the
-// table holds, or more rows than the blocks hold; and with a time limit of zero,
-// which asks for waits that run out (the cluster's hardware barrier has none).
+// table holds, or more rows than the blocks hold; and with a time limit that a
+// wait could exceed.  The hardware barriers keep none; a block reaches the next
+// one within the work on its 2400 rows, tens of microseconds, so a wait there
+// stays below any limit from kSmallLimit up.
+constexpr unsigned long long kSmallLimit = 1000000;   // 1 ms
 static int small_cluster(spuma_ldu_t h)
 {
-    if (barrier_timeout_ns() == 0) return 0;
+    if (barrier_timeout_ns() < kSmallLimit) return 0;
     if (h->ell_w < 1 || h->ell_w > 6 || h->nlev > kSmallLevels || h->n > kSmallMaxRows) return 0;
     return h->n <= kSmallOneBlock ? 1 : kSmallMaxCluster;
 }
