@@ -83,22 +83,56 @@ __global__ void k_blink(int nb, const int* __restrict__ bcell, const int8_t* __r
         if (btype[b] == 1) next[b] = atomicExch(head + bcell[b], b);
 }
 
-// d plus a_b of the cell's Dirichlet faces in ascending face order.
-__device__ __forceinline__ double add_boundary(double d, int i, const int* head, const int* next, const double* c,
+// A list in ascending order, by its cell's thread alone (bottom-up merges of
+// runs of 1, 2, 4, ... faces).
+__device__ __noinline__ int sort_list(int first, int* next)
+{
+    for (int run = 1;; run *= 2) {
+        int head = -1, tail = -1, p = first, merges = 0;
+        while (p >= 0) {
+            int q = p, np = 0, nq = run;
+            while (np < run && q >= 0) {
+                q = next[q];
+                np++;
+            }
+            merges++;
+            while (np > 0 || (nq > 0 && q >= 0)) {
+                const bool left = np > 0 && (nq == 0 || q < 0 || p < q);
+                const int e = left ? p : q;
+                if (left) {
+                    p = next[p];
+                    np--;
+                } else {
+                    q = next[q];
+                    nq--;
+                }
+                if (tail >= 0)
+                    next[tail] = e;
+                else
+                    head = e;
+                tail = e;
+            }
+            p = q;
+        }
+        next[tail] = -1;
+        first = head;
+        if (merges == 1) return first;
+    }
+}
+
+// d plus a_b of the cell's Dirichlet faces in ascending face order, a list of
+// more than one face sorted first.
+__device__ __forceinline__ double add_boundary(double d, int i, const int* head, int* next, const double* c,
                                                const double* bsf, const double* bcf, const double* bgamma)
 {
-    const int first = head ? head[i] : -1;
-    for (int last = -1; first >= 0;) {
-        int b = 0x7fffffff;
-        for (int k = first; k >= 0; k = next[k])
-            if (k > last && k < b) b = k;
-        if (b == 0x7fffffff) break;
+    int b = head ? head[i] : -1;
+    if (b >= 0 && next[b] >= 0) b = sort_list(b, next);
+    for (; b >= 0; b = next[b]) {
         const double* s = bsf + 3 * (size_t)b;
         const double* cb = bcf + 3 * (size_t)b;
         const double* ci = c + 3 * (size_t)i;
         d = __dadd_rn(d, face_coeff(s[0], s[1], s[2], __dsub_rn(cb[0], ci[0]), __dsub_rn(cb[1], ci[1]),
                                     __dsub_rn(cb[2], ci[2]), bgamma[b]));
-        last = b;
     }
     return d;
 }
@@ -108,7 +142,7 @@ __device__ __forceinline__ double add_boundary(double d, int i, const int* head,
 // ascending order.
 __global__ void k_diag(int n, const int* __restrict__ lo_start, const int* __restrict__ lo_face,
                        const int* __restrict__ own_start, const double* __restrict__ upper,
-                       const int* __restrict__ head, const int* __restrict__ next, const double* __restrict__ c,
+                       const int* __restrict__ head, int* __restrict__ next, const double* __restrict__ c,
                        const double* __restrict__ bsf, const double* __restrict__ bcf,
                        const double* __restrict__ bgamma, double* __restrict__ diag)
 {
@@ -126,7 +160,7 @@ __global__ void k_diag(int n, const int* __restrict__ lo_start, const int* __res
 template <int W>
 __global__ void __launch_bounds__(256, 8) k_diag_fl(int n, int w, const int* __restrict__ FL,
                                                     const double* __restrict__ upper, const int* __restrict__ head,
-                                                    const int* __restrict__ next, const double* __restrict__ c,
+                                                    int* __restrict__ next, const double* __restrict__ c,
                                                     const double* __restrict__ bsf, const double* __restrict__ bcf,
                                                     const double* __restrict__ bgamma, double* __restrict__ diag)
 {
