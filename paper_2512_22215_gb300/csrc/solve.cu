@@ -739,9 +739,14 @@ struct BwdR {
 
 // Levels from .. to-1 ascending (FWD) or to-1 .. from descending, one grid
 // barrier after each (after the last one too unless !last_sync).  SOLO: the
-// calling block takes whole levels by itself, with block barriers.  `at_last`
-// runs before the last level's barrier (a reduction's partials).
-template <class T, bool FWD, bool SOLO, class GR, class Op, class Last>
+// calling block takes whole levels by itself, with block barriers.  LONG: rows
+// of more than G entries are met; their entries past the first G, which the loads
+// ahead don't hold, come in groups of three (one by one, each a column and then
+// its gather, a row of 14 neighbours cost 126^3 142 against 131 ms in the mixed
+// solve; groups of six spill).  The other meshes' loop is free of that code, which
+// cost 200^3 1.6 %.  `at_last` runs before the last level's barrier (a reduction's
+// partials).
+template <class T, bool FWD, bool SOLO, bool LONG, class GR, class Op, class Last>
 __device__ __forceinline__ bool wide_sweep(const SolveArgs& a, const Mat<T>& A, const GR& g, PhaseClock& pc, int from,
                                            int to, bool last_sync, const Op& op, Last at_last)
 {
@@ -840,9 +845,11 @@ __device__ __forceinline__ bool wide_sweep(const SolveArgs& a, const Mat<T>& A, 
 #pragma unroll
                 for (int j = 0; j < G; j++)
                     if (q.c[k][j] >= 0) acc = fmadd(-q.cf[k][j], x[k][j], acc);
-                for (int j = G; j < q.e1[k] - q.e0[k]; j++) {   // rows of more than G entries
-                    const int e = FWD ? q.e0[k] + j : q.e1[k] - 1 - j;
-                    acc = fmadd(-__ldcs(coef + e), op.vec()[__ldcs(col + e)], acc);
+                if (LONG && q.e1[k] - q.e0[k] > G) {   // the rest of a longer row
+                    T rest[1] = {acc};
+                    const int b0[1] = {FWD ? q.e0[k] + G : q.e0[k]}, b1[1] = {FWD ? q.e1[k] : q.e1[k] - G};
+                    rows_chain<T, 1, 3, !FWD, true>(rest, b0, b1, col, coef, op.vec());
+                    acc = rest[0];
                 }
                 const int p = cur.pb + k * stride;
                 if (p < cur.c1) op.store(p, acc, q.s[k], L);
@@ -914,7 +921,9 @@ __device__ __forceinline__ bool sweep_levels(const SolveArgs& a, const Mat<T>& A
                                              int to, bool last_sync, const Op& op, Last at_last)
 {
     if constexpr (GR::wide) {
-        return wide_sweep<T, FWD, false>(a, A, g, pc, from, to, last_sync, op, at_last);
+        if (A.ell_w > 0 && A.ell_w <= WideShape<T>::G)
+            return wide_sweep<T, FWD, false, false>(a, A, g, pc, from, to, last_sync, op, at_last);
+        return wide_sweep<T, FWD, false, true>(a, A, g, pc, from, to, last_sync, op, at_last);
     } else {
         const RowIter it = rows_of(g);
         const int Lend = FWD ? to : from - 1;
@@ -943,7 +952,7 @@ __device__ __forceinline__ void sweep_solo(const SolveArgs& a, const Mat<T>& A, 
                                            int to, const Op& op)
 {
     if constexpr (GR::wide) {
-        wide_sweep<T, FWD, true>(a, A, g, pc, from, to, true, op, [] {});
+        wide_sweep<T, FWD, true, true>(a, A, g, pc, from, to, true, op, [] {});
     } else {
         for (int L = FWD ? from : to - 1; L != (FWD ? to : from - 1); L += FWD ? 1 : -1) {
             level_rows<T, FWD>(A, op, a.lvl[L], a.lvl[L + 1], (int)threadIdx.x, (int)blockDim.x, L);

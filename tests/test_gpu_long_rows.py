@@ -38,3 +38,39 @@ def test_caller_order_amul_bitwise():
         a = [t.astype(dt) for t in (diag, upper, x)]
         y = M.amul(*(dev(t) for t in a)).cpu().numpy()
         assert np.array_equal(bits(y), bits(oracle.amul(lo, up, *a)))
+
+
+@pytest.mark.parametrize("threads", [0, 64, 256, 512, 1024])
+def test_solves_at_matched_iterations(threads):
+    from paper_2512_22215_gb300 import LduMesh, SolverControls
+    n, lo, up, upper, diag, rng = mesh_with_rows()
+    M, b = LduMesh(lo, up, n), rng.standard_normal(n)
+    x, p = M.solve(dev(diag), dev(upper), dev(b), None,
+                   SolverControls(precond=2, tolerance=0.0, max_iter=12, block_threads=threads))
+    xo, _ = oracle.pcg(lo, up, diag, upper, b, precond=2, tol=0.0, max_iter=12)
+    assert p["status"] == 0 and p["n_iter"] == 12
+    assert np.linalg.norm(x.cpu().numpy() - xo) <= 1e-10 * np.linalg.norm(xo)
+    x, p = M.solve(dev(diag), dev(upper), dev(b), None,
+                   SolverControls(precond=2, precision=1, tolerance=1e-10, block_threads=threads))
+    r = b - oracle.amul(lo, up, diag, upper, x.cpu().numpy())
+    assert p["status"] == 0 and p["converged"] == 1 and np.abs(r).sum() <= 1e-10 * 2 * np.abs(b).sum()
+
+
+@pytest.mark.parametrize("threads", [0, 64, 1024])
+def test_preconditioner_bitwise(threads):
+    """Row order is the sequential sweeps' (through the preconditioner call, 0) and does not depend on the block size."""
+    from paper_2512_22215_gb300 import LduMesh, SolverControls
+    n, lo, up, upper, diag, rng = mesh_with_rows()
+    M, b = LduMesh(lo, up, n), rng.standard_normal(n)
+    rD, _ = oracle.dic_factor(lo, up, diag, upper)
+    if threads == 0:
+        M.prepare(dev(diag), dev(upper), 2)
+        assert np.array_equal(bits(M.read_rD().cpu().numpy()), bits(rD))
+        assert np.array_equal(bits(M.precondition(dev(b), 2).cpu().numpy()), bits(oracle.dic_precondition(lo, up, upper, rD, b)))
+        return
+    # one iteration from 0: x = alpha w
+    x, _ = M.solve(dev(diag), dev(upper), dev(b), None,
+                   SolverControls(precond=2, tolerance=0.0, max_iter=1, block_threads=threads))
+    w = oracle.dic_precondition(lo, up, upper, rD, b)
+    alpha = x.cpu().numpy()[0] / w[0]
+    assert np.abs(x.cpu().numpy() - alpha * w).max() <= 1e-13 * np.abs(alpha * w).max()
