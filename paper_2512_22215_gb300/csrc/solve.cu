@@ -648,8 +648,9 @@ __device__ __forceinline__ void level_chunk(const int* lvl, int L, int nblocks, 
 }
 
 // This block's chunks of the first kChunkTable levels, in shared memory, filled
-// once per launch (fill_chunk_table) for the wide sweeps.
-constexpr int kChunkTable = 256;
+// once per launch (fill_chunk_table) for the wide sweeps (8 KB; with 256 levels,
+// a natural order of 128^3, 382 levels, took 4.8 ms an iteration against 2.1).
+constexpr int kChunkTable = 1024;
 __device__ __forceinline__ int2* chunk_table()
 {
     __shared__ int2 table[kChunkTable];
@@ -680,6 +681,18 @@ struct WideShape {
     static constexpr int R = sizeof(T) == 4 ? 2 : 1;   // rows per thread and round
     static constexpr int G = 6;
 };
+
+// A thread without a row in a level goes on to its next one, but looks at most
+// this many levels ahead at a time and takes an empty round there: threads at the
+// edge of their block's chunks looked through all the levels left, at one step
+// while the others waited for them, which on meshes of many levels (a natural
+// order) cost more than the loads ahead gained.  An iteration, all levels | 8 | 4 |
+// 2 | none: natural 64^3 (190 levels) FP64 1288 | 1012 | 983 | 995 | 1069 us, mixed
+// 1267 | 893 | 849 | 839 | 989; 64^3 permuted (20 levels) FP64 130 | 131 | 130 | 132
+// | 142, mixed 105 | 104 | 103 | 103 | 114 (an empty round per level occupies the
+// warps that others wait beside).  One block's levels are narrower, and what an
+// empty round costs there less: 100 x 100 x 4, mixed, 468 at 4, 437 at 2.
+constexpr int kLookAhead = 4, kLookAheadSolo = 2;
 
 // The thread's rounds: row pb (and pb + stride ...) of level L, below c1.
 struct RoundIter {
@@ -763,9 +776,12 @@ __device__ __forceinline__ bool wide_sweep(const SolveArgs& a, const Mat<T>& A, 
     const T* coef = FWD ? A.Lc : A.Uc;
     const unsigned long long pol = keep_policy<T, true>();
     const int Lbeg = FWD ? from : to - 1, Lend = FWD ? to : from - 1;
-    auto open = [&](RoundIter& it) {   // first round of level it.L, or of the next level that has one
+    // first round of level it.L or of the next level that has one, kAhead levels
+    // on at most: there an empty one (see kLookAhead)
+    constexpr int kAhead = SOLO ? kLookAheadSolo : kLookAhead;
+    auto open = [&](RoundIter& it) {
         if (tid < 0) it.L = Lend;
-        while (it.L != Lend) {
+        for (int k = 0; it.L != Lend; k++) {
             int c0;
             if (chunks && it.L < kChunkTable) {
                 c0 = table[it.L].x;
@@ -777,7 +793,7 @@ __device__ __forceinline__ bool wide_sweep(const SolveArgs& a, const Mat<T>& A, 
                 it.c1 = a.lvl[it.L + 1];
             }
             it.pb = c0 + first;
-            if (it.pb < it.c1) return;
+            if (it.pb < it.c1 || k == kAhead) return;
             it.L += FWD ? 1 : -1;
         }
     };
@@ -2395,23 +2411,6 @@ int solve_blocks_per_sm(int threads, bool batch, int kind, size_t dyn = 0)
     return nb;
 }
 
-// Threads per block of a single-system solve (block_threads 0).  Up to 512 the
-// kernels have 128 registers per thread and keep a round of sweep loads in
-// flight across the grid barriers (wide_sweep).  Measured per iteration, DIC
-// FP64 / mixed, 256 | 512 | 1024 threads: 24^3 73 / 63 | 76 / 64 | 92 / 82 us,
-// 32^3 80 / 69 | 84 / 73 | 104 / 93, 64^3 119 / 98 | 112 / 92 | 151 / 131,
-// 100^3 175 / 114 | 171 / 110 | 195 / 153, 128^3 257 / 149 | 251 / 146 | 274 /
-// 174, 200^3 709 / 333 | 692 / 330 | 702 / 336; diagonal FP64 at 64^3 24 against
-// 30, at 128^3 90 against 96.  PBiCG, whose sweeps run without the loads ahead,
-// wants more threads on large meshes: DILU at 64^3 158 against 183, at 128^3 393
-// against 379.
-int default_threads(const spuma_solver_controls* ctl, int64_t n, bool bicg = false)
-{
-    if (ctl && ctl->block_threads > 0) return ctl->block_threads;
-    if (n <= 50000) return 256;
-    return bicg && n > 1000000 ? 1024 : 512;
-}
-
 // Blocks of the persistent single-system solver: one per row chunk of
 // `threads` rows, at most all co-resident blocks (SPUMA_SOLVE_BLOCKS_PER_SM
 // caps the blocks per SM, a tuning override).  0 when the kernel cannot be
@@ -2429,17 +2428,51 @@ int solve_grid(spuma_ldu_t h, int threads, int kind, size_t dyn)
     return (int)std::max<int64_t>(1, std::min<int64_t>(want, maxg));
 }
 
-// First level of the run of small last levels (each with at most `threads`
-// rows) that the solver's first block handles alone; SPUMA_TAIL_ROWS
-// overrides the row limit (0 disables).
-int tail_level(spuma_ldu_t h, int threads)
+// First level of the run of small last levels (each with at most `limit` rows)
+// that the solver's first block handles alone; SPUMA_TAIL_ROWS overrides the
+// limit (0 disables).  The limit is the block's threads, and in the DIC solves
+// at least tail_rows: a block of 256 threads takes 1024 rows in fewer steps than
+// a grid barrier costs.  Mixed, 256 threads, 256 | 512 | 1024 rows: 16^3 permuted
+// 61 | 45 | 44 us an iteration, 20^3 67 | 64 | 58, 32^3 81 | 78 | 77; FP64, whose
+// rows the pipe takes longer for, 36^3 99.5 | 99.5 | 103.
+static int tail_rows(int kind, int precision)
 {
-    int limit = threads;
+    return kind == KIND_PBICG ? 0 : precision == SPUMA_F64 ? 512 : 1024;
+}
+int tail_level(spuma_ldu_t h, int limit)
+{
     if (const char* e = getenv("SPUMA_TAIL_ROWS")) limit = atoi(e);
     int t = h->nlev;
     while (t > 1 && (int64_t)h->h_lvl[t] - h->h_lvl[t - 1] <= limit) t--;
     // keep at least two levels in the tail, else the single grid barrier saves nothing
     return (h->nlev - t >= 2) ? t : h->nlev;
+}
+
+// Threads per block of a single-system solve (block_threads 0).  Up to 512 the
+// kernels have 128 registers per thread and keep a round of sweep loads in
+// flight across the grid barriers (wide_sweep).  Measured per iteration, DIC
+// FP64 / mixed, 256 | 512 | 1024 threads: 24^3 73 / 63 | 76 / 64 | 92 / 82 us,
+// 32^3 80 / 69 | 84 / 73 | 104 / 93, 64^3 119 / 98 | 112 / 92 | 151 / 131,
+// 100^3 175 / 114 | 171 / 110 | 195 / 153, 128^3 257 / 149 | 251 / 146 | 274 /
+// 174, 200^3 709 / 333 | 692 / 330 | 702 / 336; diagonal FP64 at 64^3 24 against
+// 30, at 128^3 90 against 96.  PBiCG, whose sweeps run without the loads ahead,
+// wants more threads on large meshes: DILU at 64^3 158 against 183, at 128^3 393
+// against 379.
+// Systems that the first block has to itself past level 0 (no wider level): FP64
+// beyond one row per thread of 256 in blocks of 1024 (100 x 100 x 4, levels of 400
+// rows: 681 | 599 | 561), mixed beyond three rounds in blocks of 512 (50 x 50 x 20,
+// 970 rows: 361 | 307; below, 28^3, 588 rows: 191 | 212).
+static int default_threads(spuma_ldu_t h, const SolveArgs& a, const spuma_solver_controls* ctl)
+{
+    if (ctl->block_threads > 0) return ctl->block_threads;
+    if (a.lower_orig) return a.n <= 50000 ? 256 : a.n > 1000000 ? 1024 : 512;
+    if (a.precond == SPUMA_PRECOND_DIC && tail_level(h, 1024) <= 1) {
+        int widest = 0;
+        for (int L = 1; L < h->nlev; L++) widest = std::max(widest, h->h_lvl[L + 1] - h->h_lvl[L]);
+        if (a.precision == SPUMA_F64 && widest > 256) return 1024;
+        if (a.precision != SPUMA_F64 && widest > 768) return 512;
+    }
+    return a.n <= 50000 ? 256 : 512;
 }
 
 // The report's true residual (the solver's x in internal order is still in the
@@ -2538,7 +2571,7 @@ spuma_status launch_solve(spuma_ldu_t h, const SolveArgs& a, int threads, cudaSt
     SPUMA_CUDA(cudaMemsetAsync(h->at<char>(h->L.bar), 0, h->L.status + 256 - h->L.bar, s));
     unsigned long long tns = barrier_timeout_ns();
     SolveArgs b = a;
-    b.tail_from = tail_level(h, threads);
+    b.tail_from = tail_level(h, std::max(threads, tail_rows(kind, a.precision)));
     // SPUMA_AMUL_CHUNKS=1: the Amul phase walks level chunks when the levels
     // are wide (an average level gives every block at least a block's worth
     // of rows).  Off by default: measured at 200^3, Amul phase 101.9 -> 112.7
@@ -2627,7 +2660,7 @@ spuma_status pcg_solve_internal(spuma_ldu_t h, const double* diag, const double*
     a.perf = perf;
     spuma_status st = SPUMA_OK;
     if (ctl->block_threads != 0 || kind_of(a) != KIND_F64 || a.precond != SPUMA_PRECOND_DIC || !launch_small(h, a, s, &st))
-        st = launch_solve(h, a, default_threads(ctl, h->n), s);
+        st = launch_solve(h, a, default_threads(h, a, ctl), s);
     if (st == SPUMA_OK) h->prepared_precond = ctl->precond;
     return st;
 }
@@ -2673,7 +2706,7 @@ spuma_status spuma_pbicg_solve(spuma_ldu_t h, const double* diag, const double* 
     a.x_orig = x;
     a.perf = perf;
     h->prepared_precond = -1;
-    return launch_solve(h, a, default_threads(ctl, h->n, true), s);
+    return launch_solve(h, a, default_threads(h, a, ctl), s);
 }
 
 spuma_status spuma_matrix_prepare(spuma_ldu_t h, const double* diag, const double* upper, int32_t precond,
