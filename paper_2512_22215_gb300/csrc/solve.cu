@@ -2472,6 +2472,8 @@ static int default_threads(spuma_ldu_t h, const SolveArgs& a, const spuma_solver
         if (a.precision == SPUMA_F64 && widest > 256) return 1024;
         if (a.precision != SPUMA_F64 && widest > 768) return 512;
     }
+    // the restarted form's Amul and sweeps at 200^3, 512 | 1024 threads: 441 | 424 us an iteration (128^3 181 | 207)
+    if (a.precision == SPUMA_MIXED_RESTART && a.precond == SPUMA_PRECOND_DIC && a.n > 4000000) return 1024;
     return a.n <= 50000 ? 256 : 512;
 }
 
@@ -2800,7 +2802,11 @@ spuma_status spuma_precondition(spuma_ldu_t h, int32_t precond, const double* r,
     a.precond = precond;
     a.b_orig = r;
     a.x_orig = w;
-    return launch_solve(h, a, 256, (cudaStream_t)stream);
+    // Blocks of 256 threads with 128 registers leave too few threads an SM for the
+    // permuting passes of a large system: none, 256 | 1024 threads, 200^3 283 | 203 us,
+    // 128^3 52 | 47, 64^3 26 | 29; DIC 642 | 559, 229 | 231, 113 | 134.
+    const int large = precond == SPUMA_PRECOND_DIC ? 4000000 : 1000000;
+    return launch_solve(h, a, h->n > large ? 1024 : 256, (cudaStream_t)stream);
 }
 
 spuma_status spuma_read_phase_clocks(spuma_ldu_t h, int64_t* out, int32_t n, spuma_stream_t stream)
