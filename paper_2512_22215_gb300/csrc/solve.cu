@@ -62,9 +62,10 @@ __device__ __forceinline__ Mat<float> mat_of<float>(const SolveArgs& a)
 // in the sweeps) are loaded evict-last on top of that, and the solver hands
 // those lines back (evict-normal) before it returns; FP64 vectors, twice the
 // size, keep the default priority, since pinning them evicts them from each
-// other.  Measured at 200^3: stand-alone Amul FP64 168 -> 130 us, FP32
-// 101 -> 91 us; mixed solve 352 -> 333 ms with evict-first streams, 330 ms
-// with the FP32 gathers evict-last (FP64 gathers evict-last: Amul 130 -> 146 us).
+// other; the pipelined Amul rows gather at the default priority too.  Measured
+// at 200^3: stand-alone Amul FP64 168 -> 130 us, FP32 101 -> 91 us; mixed solve
+// 352 -> 333 ms with evict-first streams, 330 ms with the FP32 gathers evict-last
+// (FP64 gathers evict-last: Amul 130 -> 146 us).
 template <class T, bool KEEP>
 __device__ __forceinline__ unsigned long long keep_policy()
 {
@@ -113,9 +114,12 @@ struct ChainShape {
 };
 // Software-pipelined fixed-width Amul: R rows per round, whole rows of up to
 // G entries.  Where it is used was decided by measurement at 200^3: inside
-// the persistent solver for FP64 (219 -> 200 us per Amul; FP32 keeps its two
-// rows per thread in lockstep, 112 against 131 us pipelined), and in the
-// stand-alone prepared Amul for FP32 (107 -> 101 us; FP64 168 against 176 us).
+// the persistent solver for FP64 (219 -> 200 us per Amul) and, in the kernels of
+// up to 512 threads, two rows a round in both precisions (a mixed iteration with
+// the diagonal, FP32 pipelined against its two rows in lockstep: 200^3 164 | 192
+// us, 128^3 49 | 57, 64^3 20 | 20); with 1024 threads FP32 keeps the lockstep rows
+// (112 against 131 us per Amul); in the stand-alone prepared Amul for FP32 (107 ->
+// 101 us; FP64 168 against 176 us).
 template <class T>
 struct PipeShape {
     static constexpr int R = 1;
@@ -1210,13 +1214,13 @@ __device__ bool update_pass(const SolveArgs& a, Vecs<T> v, T alpha, const GR& g,
 // r -= alpha q, a pass of its own for DIC, fused into the diagonal pass
 // otherwise), whose sum|r| is handed to `after_update`: it stops the loop
 // (1), lets it go on (0) or replaces r and asks for w to be computed from the
-// new r (2).
+// new r (2).  DIC: the caller may run with the DIC preconditioner.
 // Returns 0 (w and rho ready), 2 (stop) or -1 (device error).
-template <class T, class AfterUpdate, class GR>
+template <class T, bool DIC, class AfterUpdate, class GR>
 __device__ int precondition(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, bool pending, T alpha, const GR& g,
                             PhaseClock& pc, double* rho, AfterUpdate after_update)
 {
-    if (a.precond == SPUMA_PRECOND_DIC) {
+    if (DIC && a.precond == SPUMA_PRECOND_DIC) {
         if (pending) {
             double ressum;
             if (!update_pass<T>(a, v, alpha, g, &ressum)) return -1;
@@ -1259,7 +1263,7 @@ __device__ int pcg_loop(const SolveArgs& a, const Mat<T>& A, Vecs<T> v, double n
     bool pending = false;
     for (;;) {
         rho_old = rho;
-        const int st = precondition<T>(a, A, v, pending, alpha, g, pc, &rho, [&](double ressum) {
+        const int st = precondition<T, true>(a, A, v, pending, alpha, g, pc, &rho, [&](double ressum) {
             res = ressum / nfac;
             n_it++;
             return ((n_it < max_iter && !converged(res, res0, tol, rel_tol)) || n_it < min_iter) ? 0 : 1;
@@ -1316,7 +1320,8 @@ __device__ bool refine_residual(const SolveArgs& a, const Group& g, bool fold, d
     return true;
 }
 
-// Mixed precision with reliable updates: FP32 PCG whose correction and
+// Mixed precision with reliable updates (without preconditioner or with the
+// diagonal; DIC: solve_mixed_eisenstat): FP32 PCG whose correction and
 // residual are replaced by FP64 ones (x += xs; r = b - A64 x) whenever the
 // FP32 residual has dropped by inner_rel_tol since the last replacement, the
 // FP32 residual claims convergence, or max_iter is reached; the search
@@ -1342,7 +1347,7 @@ __device__ bool solve_mixed_reliable(const SolveArgs& a, const GR& g, double nfa
         if (!group_sync(g)) return false;
         for (;;) {
             rho_old = rho;
-            const int st = precondition<float>(a, A32, v, pending, alpha, g, pc, &rho, [&](double ressum) {
+            const int st = precondition<float, false>(a, A32, v, pending, alpha, g, pc, &rho, [&](double ressum) {
                 n_it++;
                 const double ress = ressum / nfac;
                 if (!(ress < delta * rupd || converged(ress, res0, a.tol, a.rel_tol) || n_it >= a.max_iter)) return 0;
@@ -1375,8 +1380,7 @@ __device__ bool solve_mixed_reliable(const SolveArgs& a, const GR& g, double nfa
             pending = true;
         }
     }
-    // the FP32 w and p were gathered evict-last: hand their lines back
-    release_lines(a.wi, 4 * (size_t)a.n, it.first, it.stride);
+    // the Amul's rows in lockstep gather p evict-last: hand its lines back
     release_lines(a.pi, 4 * (size_t)a.n, it.first, it.stride);
     pf.initial_residual = res0;
     pf.final_residual = res;
@@ -1734,8 +1738,6 @@ __device__ bool solve_mixed_restart(const SolveArgs& a, const GR& g, double nfac
     return true;
 }
 
-// Kinds of persistent launch, one kernel each so that every kernel holds only
-// its own path (register allocation is per kernel).
 // -------------------------------------------------------------- PBiCG ---
 // One level's rows of both DILU applies (A and A^T) in one direction: they
 // share the level's structure, so the extents and columns are read once, and
@@ -2013,6 +2015,8 @@ __device__ bool solve_pbicg(const SolveArgs& a, const GR& g, double nfac, double
     return true;
 }
 
+// Kinds of persistent launch, one kernel each so that every kernel holds only
+// its own path (register allocation is per kernel).
 enum SolveKind { KIND_SETUP = 0, KIND_F64 = 1, KIND_MIXED = 2, KIND_MIXED_RESTART = 3, KIND_PBICG = 4, KIND_MIXED_DIC = 5 };
 
 }  // namespace spuma
