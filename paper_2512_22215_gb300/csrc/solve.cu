@@ -652,9 +652,10 @@ __device__ __forceinline__ void level_chunk(const int* lvl, int L, int nblocks, 
 }
 
 // This block's chunks of the first kChunkTable levels, in shared memory, filled
-// once per launch (fill_chunk_table) for the wide sweeps (8 KB; with 256 levels,
-// a natural order of 128^3, 382 levels, took 4.8 ms an iteration against 2.1).
-constexpr int kChunkTable = 1024;
+// once per launch (fill_chunk_table) for the wide sweeps.  4 KB leaves blocks of
+// 32 threads their 16 per SM; with 256 levels, a natural order of 128^3 (382
+// levels) took 4.8 ms an iteration against 2.1.
+constexpr int kChunkTable = 512;
 __device__ __forceinline__ int2* chunk_table()
 {
     __shared__ int2 table[kChunkTable];

@@ -1,6 +1,6 @@
 """GPU: meshes of many DIC levels (natural order): threads without a row for
 more levels than the sweeps look ahead, more levels than the chunk table holds
-(1024), on the grid, on the first block alone and in a batch, against the
+(512), on the grid, on the first block alone and in a batch, against the
 oracle; and the default block size against the largest one, whose sweeps
 have no loads ahead."""
 import numpy as np
