@@ -33,8 +33,8 @@ PEAKS_FALLBACK = {"hbm_gbs": 6800.0}
 # bench workload by the per-iteration byte model (traffic grows with the
 # algorithmic bytes).  Valid only for the solver source it was taken with
 # (checked by hash, else the line reports null).
-TRAFFIC = {"solve_cu_sha1": "b6798d6b171cc9be79cdaa9c0490dba6469f33d1", "n": 128,
-           "bytes": 124937681920 + 2498494208, "inner": 524, "outer": 4}
+TRAFFIC = {"solve_cu_sha1": "3c656a00ddefa4fcbcc9bf8000155beadadc2eba", "n": 128, "iteration": "it32_eisenstat",
+           "bytes": 74949389056 + 927484416, "inner": 522, "outer": 5}
 # Iteration counts of this seeded workload (mixed: inner iterations, outer
 # steps), used only to project the CPU oracle's bounded sample to a full solve.
 PROJECTION_ITERS = {"inner": 795, "outer": 5}
@@ -99,18 +99,20 @@ def traffic_bytes(n_cells: int, n_faces: int, inner: int, outer: int):
     n = TRAFFIC["n"]
     nf = 3 * (n - 1) * n * n
     wc, wb = workload_bytes(n ** 3, nf), workload_bytes(n_cells, n_faces)
-    cap = TRAFFIC["inner"] * wc["it32"] + (TRAFFIC["outer"] + 1) * wc["resid64"]
-    this = inner * wb["it32"] + (outer + 1) * wb["resid64"]
+    it = TRAFFIC.get("iteration", "it32")
+    cap = TRAFFIC["inner"] * wc[it] + (TRAFFIC["outer"] + 1) * wc["resid64"]
+    this = inner * wb[it] + (outer + 1) * wb["resid64"]
     return int(TRAFFIC["bytes"] * this / cap)
 
 
 def workload_bytes(n_cells: int, n_faces: int):
     """Algorithmic bytes (LDU basis, int32 indices) of one PCG iteration and of
-    one Amul: FP64 iteration 152N + 48F, FP32 iteration 76N + 36F, FP64 Amul
+    one Amul: FP64 iteration 152N + 48F, FP32 iteration 76N + 36F with its Amul
+    and 72N + 16F in Eisenstat's form (what the mixed DIC solve runs), FP64 Amul
     16F + 24N, FP32 Amul 12F + 12N, FP64 residual b - A x 16F + 40N."""
     N, F = n_cells, n_faces
-    return dict(it64=152 * N + 48 * F, it32=76 * N + 36 * F, amul64=16 * F + 24 * N, amul32=12 * F + 12 * N,
-                resid64=16 * F + 40 * N)
+    return dict(it64=152 * N + 48 * F, it32=76 * N + 36 * F, it32_eisenstat=72 * N + 16 * F,
+                amul64=16 * F + 24 * N, amul32=12 * F + 12 * N, resid64=16 * F + 40 * N)
 
 
 def parse_cpulist(text: str) -> set:
@@ -725,7 +727,7 @@ def main():
     wb = workload_bytes(N, F)
     peaks, peak_kind = load_peaks()
     hbm = float(peaks.get("hbm_gbs", PEAKS_FALLBACK["hbm_gbs"]))
-    mixed_bytes = p_mixed["n_iter"] * wb["it32"] + (p_mixed["n_outer"] + 1) * wb["resid64"]
+    mixed_bytes = p_mixed["n_iter"] * wb["it32_eisenstat"] + (p_mixed["n_outer"] + 1) * wb["resid64"]
     achieved = mixed_bytes / (solve_mixed_ms * 1e-3) / 1e9
     f64_bytes = p_f64["n_iter"] * wb["it64"]
     roofline = {"kernel": "k_solve (persistent mixed-precision solve, one launch per solve)", "bound": "hbm",
@@ -733,7 +735,7 @@ def main():
                 "peak_kind": peak_kind,
                 "traffic": traffic_bytes(N, F, p_mixed["n_iter"], p_mixed["n_outer"]),
                 "algorithmic_bytes": int(mixed_bytes),
-                "basis": "inner iterations x (76N + 36F) + (outer + 1) FP64 residuals x (16F + 40N)"}
+                "basis": "inner iterations x (72N + 16F) + (outer + 1) FP64 residuals x (16F + 40N)"}
 
     line = {
         "metric": METRIC, "value": round(ms_step_max, 3), "unit": "ms", "n_gpus": world, "steps": args.steps,
