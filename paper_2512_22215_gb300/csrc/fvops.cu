@@ -271,9 +271,9 @@ __global__ void __launch_bounds__(256, 8) k_fv_cell_sum_fl(int n, int w, const i
 // corr_f = (gamma_f |S|) (k . (w grad_l + (1 - w) grad_u)), k = S/|S| - d delta,
 // delta = 1/max(n.d, 0.05 |d|) (the implicit part's coefficient).
 // dcp_f = corr_f - phi_f as well, the face term of the right-hand side.
-// Bound by the FP64 pipe (86 % active): 63 instructions a face with one
-// reciprocal for the four quotients by |S| and one for delta (110 with the
-// built-in operations); with the cell sum, 2.2M cells: 1277 -> 933 us.
+// Bound by the FP64 pipe (86 % active): 68 instructions a face (by time and
+// pipe activity) with one reciprocal for the four quotients by |S| and one for
+// delta, 98 with the built-in operations; with the cell sum, 2.2M cells: 1277 -> 933 us.
 __global__ void k_fv_corr(int nf, const int* __restrict__ l, const int* __restrict__ u,
                           const double* __restrict__ sf, const double* __restrict__ c,
                           const double* __restrict__ w, const double* __restrict__ gamma,

@@ -20,10 +20,10 @@ static int grid1d(int64_t work, int threads, int num_sms)
     return (int)std::max<int64_t>(g, 1);
 }
 
-// upper_f = -a_f in face order.  Bound by the FP64 pipe: about 38 instructions
-// a face with the shared reciprocals of fp64.cuh (60 with the built-in
-// division and square root): 200^3 assembly 2.87 -> 2.05 ms, its reverse mode
-// 2.49 -> 1.62 ms.
+// upper_f = -a_f in face order.  Bound by the FP64 pipe: about 35 instructions
+// a face (by time and pipe activity, 87 %) with the shared reciprocals of
+// fp64.cuh, 54 with the built-in division and square root: 200^3 assembly 2.87 ->
+// 2.05 ms, its reverse mode 2.49 -> 1.62 ms.
 __global__ void k_face_coeff(int nf, const int* __restrict__ l, const int* __restrict__ u,
                              const double* __restrict__ sf, const double* __restrict__ c,
                              const double* __restrict__ gamma, double* __restrict__ upper)
