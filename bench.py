@@ -33,8 +33,8 @@ PEAKS_FALLBACK = {"hbm_gbs": 6800.0}
 # bench workload by the per-iteration byte model (traffic grows with the
 # algorithmic bytes).  Valid only for the solver source it was taken with
 # (checked by hash, else the line reports null).
-TRAFFIC = {"solve_cu_sha1": "3c656a00ddefa4fcbcc9bf8000155beadadc2eba", "n": 128, "iteration": "it32_eisenstat",
-           "bytes": 74949389056 + 927484416, "inner": 522, "outer": 5}
+TRAFFIC = {"solve_cu_sha1": "e0190969ad9957e142035f9b1dbf231d48c9acd8", "n": 128, "iteration": "it32_eisenstat",
+           "bytes": 74956187648 + 933906944, "inner": 522, "outer": 5}
 # Iteration counts of this seeded workload (mixed: inner iterations, outer
 # steps), used only to project the CPU oracle's bounded sample to a full solve.
 PROJECTION_ITERS = {"inner": 795, "outer": 5}

@@ -2460,7 +2460,10 @@ int tail_level(spuma_ldu_t h, int limit)
 // 32^3 80 / 69 | 84 / 73 | 104 / 93, 64^3 119 / 98 | 112 / 92 | 151 / 131,
 // 100^3 175 / 114 | 171 / 110 | 195 / 153, 128^3 257 / 149 | 251 / 146 | 274 /
 // 174, 200^3 709 / 333 | 692 / 330 | 702 / 336; diagonal FP64 at 64^3 24 against
-// 30, at 128^3 90 against 96.  PBiCG, whose sweeps run without the loads ahead,
+// 30, at 128^3 90 against 96; mixed with the diagonal, 256 or 512 by this rule |
+// 1024: 24^3 14 | 26, 48^3 18 | 26, 64^3 20 | 28, 128^3 49 | 59, 200^3 164 | 167;
+// restarted, diagonal: 13 | 25, 17 | 25, 19 | 26, 47 | 56, 160 | 160, DIC 68 | 90, 88 |
+// 116, 101 | 137, 181 | 207, 441 | 424.  PBiCG, whose sweeps run without the loads ahead,
 // wants more threads on large meshes: DILU at 64^3 158 against 183, at 128^3 393
 // against 379.
 // Systems that the first block has to itself past level 0 (no wider level): FP64
